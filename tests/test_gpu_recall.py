@@ -41,6 +41,31 @@ def test_hits_match_the_oracle(vie, n, k, m):
     np.testing.assert_array_equal(got.cpu().numpy(), oracle.recall_hits(ex, ap))
 
 
+@pytest.mark.parametrize("n,k,m", [
+    (300, 8, 33), (300, 9, 127),              # registers / hash table
+    (4097, 128, 130), (4097, 129, 129),       # a table per warp / per CTA
+    (5000, 100, 1025), (700, 100, 1025),      # by the number of queries
+    (50, 1000, 3), (3, 11, 1 << 17)])
+def test_hits_with_colliding_and_repeated_entries(vie, n, k, m):
+    """Exact entries whose hash slots all fall at the end of the table (long
+    probes that wrap around), a third of them repeated, and the largest int32."""
+    import torch
+    rng = np.random.default_rng(n + k)
+    slots = 64
+    while slots < 4 * k:
+        slots *= 2
+    v = np.arange(1, 400000, dtype=np.uint32)
+    hashed = (v * np.uint32(0x9E3779B1)) >> np.uint32(32 - slots.bit_length() + 1)
+    pool = np.append(v[hashed >= slots - 2], np.uint32(2**31 - 1)).astype(np.int32)
+    ex = rng.choice(pool, (n, k)).astype(np.int32)
+    ex[rng.random((n, k)) < 0.05] = -1
+    ap = rng.choice(np.concatenate([pool, np.arange(-2, 200, dtype=np.int32)]), (n, m)).astype(np.int32)
+    got = vie.recall_hits(torch.from_numpy(ex).cuda(), torch.from_numpy(ap).cuda())
+    torch.cuda.synchronize()
+    rows = np.arange(n) if n * k * m < 2e8 else np.arange(0, n, 5)
+    np.testing.assert_array_equal(got.cpu().numpy()[rows], oracle.recall_hits(ex[rows], ap[rows]))
+
+
 def test_hits_edge_lists(vie):
     import torch
     ex = np.arange(64, dtype=np.int32).reshape(2, 32)
