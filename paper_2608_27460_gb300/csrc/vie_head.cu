@@ -677,6 +677,7 @@ static vie_status run_topk(const char *fn, vie_head *head, const float *h, int32
                                 head->d_pad * (head->scale != nullptr ? 1 : 2), p.sel_cap);
         const uint32_t early_bytes = vie::SmemLayout::merge_fixed_bytes() + 8u * vie::kFastE * head->G +
                                      4u * ((head->G + 7) & ~7);
+        p.pdl = 1;  // the handle's W never changes
         p.early = (opt(VIE_OPT_EARLY_MERGE) != 0 && nq == 1 && k <= vie::kFastMaxK && head->G >= 2 &&
                    2 * head->G <= vie::kThreads && L.total - L.merge >= early_bytes) ? 1 : 0;
         // several queries: the first CTAs to finish merge them in parallel
@@ -1081,6 +1082,7 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
         p.ticket = counters;
         p.next_chunk = counters + 2;
         p.err = nd.flag;
+        p.pdl = 0;    // the caller's W may come from the kernel before this one
         p.early = 0;  // the last-ticket merge: no per-CTA words in the fixed array
         p.pmerge = 0;
         p.epoch = nullptr;

@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(128) sample_topk_kernel(const int32_t *__restr
                                                          float min_p, uint64_t seed, uint64_t step,
                                                          int32_t *__restrict__ out_token,
                                                          float *__restrict__ out_prob) {
+    griddep_launch_dependents();  // the next head launch may start streaming its weights
     griddep_wait();  // the candidates may come from the kernel before this one
     const int lane = threadIdx.x & 31;
     const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);

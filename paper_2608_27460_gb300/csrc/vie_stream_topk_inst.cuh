@@ -19,8 +19,17 @@ cudaError_t launch_one(const StreamTopkParams &p, int grid, uint32_t smem, cudaS
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    stream_topk_kernel<NB, MM, kR, Q8><<<grid, threads_for<NB>(), smem, stream>>>(p);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(threads_for<NB>());
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p.pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, stream_topk_kernel<NB, MM, kR, Q8>, p);
 }
 
 template <int NB, int R, bool Q8>
