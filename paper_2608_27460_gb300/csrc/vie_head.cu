@@ -65,7 +65,7 @@ struct vie_head {
     int G;
     uint16_t *W;        // [V, d_pad] bf16 bits, or e4m3 codes (bytes) when scale is set
     float *scale;       // e4m3 heads: fp32 scale per row [V]; nullptr for bf16 heads
-    uint64_t *cand;     // [kMaxNB][G][VIE_K_MAX] ranking keys, then [kMaxNB][G][kFastE] heads
+    uint64_t *cand;     // [kMaxNB][G][VIE_K_MAX] ranking keys, then [kMaxNB][G][kWideE] heads
     uint32_t *words;    // kNumWords scratch words (see kEpochWord, kFlagWords)
     int64_t scratch_bytes;
     // tensor-core path (batches): hi/lo bf16 query matrix and TMA descriptors
@@ -176,17 +176,26 @@ __global__ void scatter_sparse_kernel(const int32_t *__restrict__ idx,
 // ---------------------------------------------------------------------------
 namespace {
 
-// Selector of the streaming kernel: register lists of 2 keys per lane for
-// k <= 64, else (0) the shared-memory candidate buffers of the wide lists.
-int pick_mm(int k) { return k <= vie::kFastMaxK ? 2 : 0; }
+// Selector of the streaming kernel: register lists of 2 keys per lane (2), or
+// the shared-memory candidate buffers (0): for k > 64, and for k <= 64 where a
+// CTA's share of W is so short (rows x row_bytes up to kBufSelBytes, ~15 us of
+// its stream) that the register lists' insertions (k (1 + ln(rows / k)) keys
+// at ~0.14 us) would outlast it.
+constexpr int64_t kBufSelBytes = 640 * 1024;
+int pick_mm(int k, int64_t V, int G, int row_bytes) {
+    if (k > vie::kFastMaxK) return 0;
+    return (V + G - 1) / G * row_bytes <= kBufSelBytes ? 0 : 2;
+}
 
-// Keys per query of a launch's candidate buffers (wide lists): a single
-// query gets about 4k (its first cut-back comes early in the stream, where it
-// is hidden, and usually stays the only one; the CTA's final selection then
-// sorts a few k keys, not every row it streamed), groups the least size for k.
-int sel_cap_launch(int nb, int k) {
+// Keys per query of a launch's candidate buffers: for k <= 64 a size whose
+// keys one CTA ranks by counting; for wide lists a single query gets about 4k
+// (its first cut-back comes early in the stream, where it is hidden, and
+// usually stays the only one), groups the least size for k.
+int sel_cap_launch(int mm, int nb, int k) {
+    if (mm != 0) return 0;
+    if (k <= vie::kFastMaxK) return vie::kSelCapFast;
     const int c = vie::sel_cap_for(k);
-    if (nb != 1 || c == 0) return c;
+    if (nb != 1) return c;
     const int c4 = (4 * k + 63) & ~63;
     return c4 > kMaxSelBytes / 8 ? kMaxSelBytes / 8 : c4;
 }
@@ -249,19 +258,21 @@ struct LaunchShape {
 };
 
 // Rows per warp per stage (R), stage rows (8*R, fewer for very wide rows),
-// and ring depth (deepest that fits) for one launch.
-bool pick_shape(int nb, int d_pad, int row_bytes, int sel_cap, LaunchShape *out) {
+// and ring depth (deepest that fits) for one launch, whose merge may need
+// merge_bytes of the ring's shared memory.
+bool pick_shape(int nb, int d_pad, int row_bytes, int sel_cap, uint32_t merge_bytes, LaunchShape *out) {
     const int r_max = nb == 1 ? 8 : 4;  // 8 rows per warp only for single-query launches
     int r = 1;
     while (r < r_max && 8 * r * row_bytes < opt(VIE_OPT_STAGE_MIN_KB) * 1024) r <<= 1;
     for (int rs = 8 * r; rs >= 1; --rs) {
         for (int s = vie::kMaxStages; s >= 2; --s) {
             const vie::SmemLayout L(nb, d_pad, rs, s, row_bytes, sel_cap);
-            if (L.total <= static_cast<uint32_t>(kMaxSmem)) {
+            const uint32_t total = L.total > L.merge + merge_bytes ? L.total : L.merge + merge_bytes;
+            if (total <= static_cast<uint32_t>(kMaxSmem)) {
                 out->r = r;
                 out->rs = rs;
                 out->stages = s;
-                out->smem = L.total;
+                out->smem = total;
                 return true;
             }
         }
@@ -400,7 +411,7 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
 
     const size_t wbytes = static_cast<size_t>(V) * hd->d_pad * (e4m3 ? 1 : 2);
     const size_t cbytes =
-        static_cast<size_t>(kMaxNB) * hd->G * (VIE_K_MAX + vie::kFastE) * sizeof(uint64_t);
+        static_cast<size_t>(kMaxNB) * hd->G * (VIE_K_MAX + vie::kWideE) * sizeof(uint64_t);
     hd->scratch_bytes = static_cast<int64_t>(cbytes + kNumWords * sizeof(uint32_t));
     e = cudaMalloc(&hd->W, wbytes);
     if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->scale, static_cast<size_t>(V) * sizeof(float));
@@ -637,17 +648,21 @@ static vie_status run_topk(const char *fn, vie_head *head, const float *h, int32
     vie_status st = check_device(head);
     if (st != VIE_OK) return st;
 
-    const int mm = pick_mm(k);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (use_tc(head, batch, k)) return run_topk_tc(fn, head, h, batch, k, out_idx, out_logits, sparse, s);
+    const int row_bytes = head->d_pad * (head->scale != nullptr ? 1 : 2);
+    const int mm = pick_mm(k, head->V, head->G, row_bytes);
+    // published wide lists: the merge stages kWideE keys of every list
+    const bool wide = k > vie::kFastMaxK && head->G <= vie::kThreads;
+    const uint32_t wide_bytes = vie::SmemLayout::merge_fixed_bytes() + 8u * vie::kWideE * head->G;
     const int cap = nb_cap_for(head->d_pad, k);
     for (int q0 = 0; q0 < batch; q0 += cap) {
         const int nq = batch - q0 < cap ? batch - q0 : cap;
         int nb = 1;
         while (nb < nq) nb <<= 1;
         LaunchShape shp;
-        if (!pick_shape(nb, head->d_pad, head->d_pad * (head->scale != nullptr ? 1 : 2), sel_cap_launch(nb, k),
-                        &shp))
+        const int sel_cap = sel_cap_launch(mm, nb, k);
+        if (!pick_shape(nb, head->d_pad, row_bytes, sel_cap, wide ? wide_bytes : 0u, &shp))
             return fail(VIE_ERR_UNSUPPORTED, "%s: no shared-memory layout for d=%d", fn, head->d);
         vie::StreamTopkParams p;
         p.W = head->W;
@@ -665,7 +680,8 @@ static vie_status run_topk(const char *fn, vie_head *head, const float *h, int32
         p.static_chunks = static_cast<int32_t>(n_chunks * pct / 100 / head->G);
         p.pool_rows = pool_rows_for(shp.rs);
         p.half_rows = half_rows_for(shp.r, head->d_pad / (head->scale != nullptr ? 16 : 8));
-        p.sel_cap = sel_cap_launch(nb, k);
+        p.sel_cap = sel_cap;
+        p.list_keys = wide ? (sel_cap < VIE_K_MAX ? sel_cap : VIE_K_MAX) : k;
         p.cand = head->cand;
         p.heads = head->cand + static_cast<size_t>(kMaxNB) * head->G * VIE_K_MAX;
         p.ticket = head->words;
@@ -673,15 +689,15 @@ static vie_status run_topk(const char *fn, vie_head *head, const float *h, int32
         p.next_chunk = head->words + 2;
         // one query, k <= 64: CTA 0 merges the lists as they arrive (its
         // merge buffers and every list's first keys in the ring's shared memory)
-        const vie::SmemLayout L(nb, head->d_pad, shp.rs, shp.stages,
-                                head->d_pad * (head->scale != nullptr ? 1 : 2), p.sel_cap);
+        const vie::SmemLayout L(nb, head->d_pad, shp.rs, shp.stages, row_bytes, sel_cap);
         const uint32_t early_bytes = vie::SmemLayout::merge_fixed_bytes() + 8u * vie::kFastE * head->G +
                                      4u * ((head->G + 7) & ~7);
         p.pdl = 1;  // the handle's W never changes
         p.early = (opt(VIE_OPT_EARLY_MERGE) != 0 && nq == 1 && k <= vie::kFastMaxK && head->G >= 2 &&
-                   2 * head->G <= vie::kThreads && L.total - L.merge >= early_bytes) ? 1 : 0;
-        // several queries: the first CTAs to finish merge them in parallel
-        p.pmerge = (nq > 1 && head->G <= vie::kThreads && L.total - L.merge >= early_bytes) ? 1 : 0;
+                   2 * head->G <= vie::kThreads && shp.smem - L.merge >= early_bytes) ? 1 : 0;
+        // several queries, or wide lists: the first CTAs to finish merge them in parallel
+        p.pmerge = (wide || (nq > 1 && k <= vie::kFastMaxK && head->G <= vie::kThreads &&
+                             shp.smem - L.merge >= early_bytes)) ? 1 : 0;
         p.epoch = head->words + kEpochWord;
         p.flags = head->words + kFlagWords;
         p.out_idx = out_idx + static_cast<int64_t>(q0) * k;
@@ -1027,7 +1043,7 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
     if (g > nd.sms) g = nd.sms;
     if (g > vie::kMaxLists) g = vie::kMaxLists;
     const int G = static_cast<int>(g < 1 ? 1 : g);
-    const int mm = pick_mm(k);
+    const int mm = pick_mm(k, V, G, d * 2);
     const int cap = nb_cap_for(d, k);
     int nb_max = 1;
     while (nb_max < cap && nb_max < batch) nb_max <<= 1;
@@ -1058,7 +1074,7 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
         int nb = 1;
         while (nb < nq) nb <<= 1;
         LaunchShape shp;
-        if (!pick_shape(nb, d, d * 2, sel_cap_launch(nb, k), &shp))
+        if (!pick_shape(nb, d, d * 2, sel_cap_launch(mm, nb, k), 0u, &shp))
             return fail(VIE_ERR_UNSUPPORTED, "%s: no shared-memory layout for d=%d", fn, d);
         vie::StreamTopkParams p;
         p.W = static_cast<const uint16_t *>(W_out);
@@ -1076,7 +1092,8 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
         p.static_chunks = static_cast<int32_t>(n_chunks * pct / 100 / G);
         p.pool_rows = pool_rows_for(shp.rs);
         p.half_rows = half_rows_for(shp.r, d / 8);
-        p.sel_cap = sel_cap_launch(nb, k);
+        p.sel_cap = sel_cap_launch(mm, nb, k);
+        p.list_keys = k;
         p.cand = cand;
         p.heads = heads;
         p.ticket = counters;

@@ -81,6 +81,8 @@ constexpr int kRankCountMax = 640;     // rank counting below this many keys
 constexpr int kMaxLists = 1024;        // G <= 1024 CTAs
 constexpr int kFastE = 8;              // fast merge: entries read per list (even)
 constexpr int kFastMaxK = 64;          // fast merge: largest k
+constexpr int kWideE = 32;             // published wide lists: sorted keys per list in the heads area
+constexpr int kSelCapFast = 256;       // candidate buffer keys per query, k <= kFastMaxK
 constexpr int kSelRun = 128;           // keys of one sorted run (a warp's registers)
 constexpr int kRankRunsMin = kRankCountMax;  // merge output: a bitonic sort above this many keys
 
@@ -106,15 +108,16 @@ struct StreamTopkParams {
     int32_t static_chunks;   // chunks each CTA owns before drawing from the pool
     int32_t pool_rows;       // rows of a pool piece (<= rows_per_stage)
     int32_t half_rows;       // 1: each half-warp projects its own row (R >= 2)
-    int32_t sel_cap;         // wide lists: buffer keys per query (sel_cap_for(k)); else 0
-    uint64_t *cand;          // [NB][G][k] keys
-    uint64_t *heads;         // [NB][G][kFastE]: the first keys of each list
+    int32_t sel_cap;         // candidate buffers: keys per query; 0 with register lists
+    int32_t list_keys;       // keys of a list in cand: k, or more for published wide lists
+    uint64_t *cand;          // [NB][G][list_keys] keys
+    uint64_t *heads;         // [NB][G][kFastE] (published wide lists: kWideE): the first keys of each list
     uint32_t *ticket;        // CTA completion counter (self-resetting)
     uint32_t *next_chunk;    // pool counter (self-resetting)
     uint32_t *err;           // device flag word
     int32_t early;           // 1: CTA 0 merges the lists as they are published (nq == 1)
     int32_t pmerge;          // 1: the first min(nq, G) CTAs to finish merge the queries,
-                             //    each taking the lists as they are published (nq > 1)
+                             //    each taking the lists as they are published (nq > 1 or k > 64)
     uint32_t *epoch;         // launch counter word (early merge or pmerge)
     uint32_t *flags;         // [G] publication words (early merge or pmerge)
     int32_t *out_idx;        // [nq, k]
@@ -616,6 +619,45 @@ __device__ inline void write_cta_list(uint64_t *buf, int cnt, int k, uint32_t *h
     for (int i = m + tid; i < kFastE; i += nthr) head[i] = 0ull;
 }
 
+// The same for k <= kFastMaxK: every key of the buffer (at most kSelCapFast)
+// is ranked by counting the keys above it, one thread per key, and the best k
+// go out at their rank.  About 0.5 us for 256 keys, where a sorted register
+// list pays ~0.14 us for every key that enters it.
+__device__ inline void write_ranked_list(const uint64_t *buf, int cnt, int k, uint64_t *dst, uint64_t *head) {
+    const int tid = threadIdx.x, nthr = static_cast<int>(blockDim.x);
+    for (int i = tid; i < cnt; i += nthr) {
+        const uint64_t x = buf[i];
+        const int rank = rank_among(buf, cnt, x);
+        if (rank < k) dst[rank] = x;
+        if (rank < kFastE) head[rank] = rank < k ? x : 0ull;
+    }
+    for (int i = cnt + tid; i < k; i += nthr) dst[i] = 0ull;
+    for (int i = cnt + tid; i < kFastE; i += nthr) head[i] = 0ull;
+}
+
+// Published wide lists, one warp per query, after the stream: the buffer's
+// cnt keys (cut back to k if they are more than list_keys, which is at least
+// k) to dst, unsorted, zeros after them, and the best kWideE of them, sorted,
+// to head (zeros after the real keys).  A CTA's expected share of the top k is
+// k / G, so the merge seldom needs more of a list than its head; sorting whole
+// lists (a radix select and a block sort per query) was most of the launch's
+// tail.
+static __device__ __noinline__ void write_wide_list(uint64_t *buf, int cnt, int k, int list_keys, uint64_t *dst,
+                                                    uint64_t *head, int lane) {
+    if (cnt > list_keys) cnt = warp_cut_back(buf, cnt, k, k, lane).n;
+    __syncwarp();
+    for (int i = lane; i < list_keys; i += 32) dst[i] = i < cnt ? buf[i] : 0ull;
+    if (cnt > 2 * kWideE) cnt = warp_cut_back(buf, cnt, kWideE, 2 * kWideE, lane).n;
+    __syncwarp();
+    uint64_t v[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) v[j] = lane * 2 + j < cnt ? buf[lane * 2 + j] : 0ull;
+    warp_sort_desc<2>(v, lane);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+        if (lane * 2 + j < kWideE) head[lane * 2 + j] = v[j];
+}
+
 // Shared-memory buffers of the merge.
 struct MergeBufs {
     uint64_t *pref, *cands, *win;
@@ -976,6 +1018,105 @@ __device__ inline void merge_published(const uint32_t *flags, uint32_t target, c
         merge_lists(GlobalKeys{lists_q}, G, k, mb, ms, oi, ol, sp);
 }
 
+// Merge of one query from published wide lists (k > kFastMaxK; every thread
+// of the merging CTA, at least G threads): polls the publication words as
+// merge_published does, then
+//   1. brings the lists' heads (G x kWideE sorted keys) into shared memory;
+//   2. tau = the k-th largest key among the first J of every list (a lower
+//      bound on the k-th key, 0 if they hold fewer than k keys);
+//   3. unless some list's last head key is still >= tau (it may hold more),
+//      the exact top-k of the head keys >= tau is the answer; otherwise every
+//      key >= tau is gathered from the whole lists (lists_q, G x list_keys,
+//      unsorted, zeros as empty slots).
+// ws holds the merge buffers (merge_fixed_bytes), fe G * kWideE keys.
+__device__ inline void merge_published_wide(const uint32_t *flags, uint32_t target, const uint64_t *heads_q,
+                                            const uint64_t *lists_q, int list_keys, int G, int k,
+                                            unsigned char *ws, uint64_t *fe, MiscSmem *ms, uint32_t *err,
+                                            int32_t *oi, float *ol, float *sp) {
+    const int tid = threadIdx.x, lane = tid & 31, nthr = static_cast<int>(blockDim.x);
+    MergeBufs mb;
+    mb.pref = reinterpret_cast<uint64_t *>(ws);
+    mb.cands = mb.pref + kMergePrefixCap;
+    mb.win = mb.cands + kMergeCandCap;
+    mb.counts = reinterpret_cast<int *>(mb.win + 1024);
+    mb.offsets = mb.counts + kMaxLists;
+    mb.hist = reinterpret_cast<uint32_t *>(mb.offsets + kMaxLists);
+    if (tid == 0) {
+        ms->n_cand = 0;
+        ms->n_win = 0;
+        ms->overflow = 0;
+        ms->remaining = 0;
+    }
+    const uint64_t t0 = global_timer_ns();
+    for (bool pending = tid < G;;) {
+        if (pending) {
+            if (ld_acquire_gpu(flags + tid) == target) {
+                pending = false;
+            } else if (global_timer_ns() - t0 > kWaitLimitNs) {
+                pending = false;
+                atomicOr(err, kErrWaitTimeout);
+            }
+        }
+        if (__syncthreads_count(pending ? 1 : 0) == 0) break;
+    }
+    // 1. the heads
+    const int n_heads = G * kWideE;
+    const ulonglong2 *src2 = reinterpret_cast<const ulonglong2 *>(heads_q);
+    ulonglong2 *fe2 = reinterpret_cast<ulonglong2 *>(fe);
+#pragma unroll 4
+    for (int i = tid; i < n_heads / 2; i += nthr) fe2[i] = __ldcg(src2 + i);
+    __syncthreads();
+    // 2. tau from the first J keys of every list: twice the expected share
+    int J = (2 * k + G - 1) / G;
+    J = min(J, min(kWideE, kMergePrefixCap / G));
+    const int P = G * J;
+    int nz = 0;
+    for (int i = tid; i < P; i += nthr) {
+        const uint64_t x = fe[(i / J) * kWideE + i % J];
+        mb.pref[i] = x;
+        nz += x != 0 ? 1 : 0;
+    }
+    nz = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(nz)));
+    if (lane == 0 && nz != 0) atomicAdd(&ms->remaining, nz);
+    __syncthreads();
+    const bool enough = ms->remaining >= k;
+    __syncthreads();  // block_radix_threshold reuses the word
+    const uint64_t tau = enough ? block_radix_threshold(SmemKeys{mb.pref}, P, k, 1, mb.hist, ms) : 0;
+    const uint64_t lo = tau > 0 ? tau : 1;
+    // 3. the candidates
+    if (tid < G && fe[tid * kWideE + kWideE - 1] >= lo) ms->overflow = 1;
+    __syncthreads();
+    const bool whole = ms->overflow != 0;
+    const int n = whole ? G * list_keys : n_heads;
+    for (int i0 = tid - lane; i0 < n; i0 += nthr) {
+        const int i = i0 + lane;
+        uint64_t x = 0;
+        if (i < n) x = whole ? GlobalKeys{lists_q}[i] : fe[i];
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, x >= lo);
+        if (m == 0) continue;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&ms->n_cand, __popc(m));
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        const int pos = base + __popc(m & ((1u << lane) - 1u));
+        if (x >= lo && pos < kMergeCandCap) mb.cands[pos] = x;
+    }
+    __syncthreads();
+    const int M = ms->n_cand;
+    if (M <= kMergeCandCap) {
+        block_topk_to_output(mb.cands, M, k, mb.win, mb.hist, ms, oi, ol, sp);
+        return;
+    }
+    // too many for the buffer: the exact threshold first
+    const uint64_t T = whole ? block_radix_threshold(GlobalKeys{lists_q}, n, k, lo, mb.hist, ms)
+                             : block_radix_threshold(SmemKeys{fe}, n, k, lo, mb.hist, ms);
+    for (int i = tid; i < n; i += nthr) {
+        const uint64_t x = whole ? GlobalKeys{lists_q}[i] : fe[i];
+        if (x >= T && x >= lo) mb.win[atomicAdd(&ms->n_win, 1)] = x;
+    }
+    __syncthreads();
+    block_topk_to_output(mb.win, k, k, mb.win, mb.hist, ms, oi, ol, sp);
+}
+
 // --------------------------------------------------------------------------
 // Rows of the stage that starts at row0: whole chunks (RS rows) in the
 // round-robin part, pool pieces (RSH rows) behind it, and never past the
@@ -1191,7 +1332,16 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&sempty[s]);
                 }
-                if (lane == 0) {
+                if (p.k > kFastMaxK && p.pmerge) {
+#pragma unroll
+                    for (int j = 0; j < QPS; ++j) {
+                        const int nb = sw + j * NS;
+                        if (nb < p.nq)
+                            write_wide_list(sbuf + nb * cap, cnt[j], p.k, p.list_keys,
+                                            p.cand + (static_cast<size_t>(nb) * G + cta) * p.list_keys,
+                                            p.heads + (static_cast<size_t>(nb) * G + cta) * kWideE, lane);
+                    }
+                } else if (lane == 0) {
 #pragma unroll
                     for (int j = 0; j < QPS; ++j) ms->sel_cnt[sw + j * NS] = sw + j * NS < p.nq ? cnt[j] : 0;
                 }
@@ -1400,17 +1550,22 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
         }
     }
 
-    // ---------------- wide lists: buffers -> sorted lists ----------------
-    // (the ring is free: every stage was consumed before its role ended)
+    // ---------------- buffers -> sorted lists ----------------
+    // (the ring is free: every stage was consumed before its role ended;
+    // published wide lists have been written by the selectors already)
     if constexpr (MM == 0) {
         __syncthreads();
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + L.ring);
-        uint64_t *win = reinterpret_cast<uint64_t *>(smem + L.ring + 1024);
         uint64_t *sbuf = reinterpret_cast<uint64_t *>(smem + L.sel);
-        for (int nb = 0; nb < p.nq; ++nb)
-            write_cta_list(sbuf + nb * p.sel_cap, ms->sel_cnt[nb], p.k, hist, win, ms,
-                           p.cand + (static_cast<size_t>(nb) * G + cta) * p.k,
-                           p.heads + (static_cast<size_t>(nb) * G + cta) * kFastE);
+        for (int nb = 0; nb < p.nq; ++nb) {
+            uint64_t *buf = sbuf + nb * p.sel_cap;
+            uint64_t *dst = p.cand + (static_cast<size_t>(nb) * G + cta) * p.k;
+            uint64_t *head = p.heads + (static_cast<size_t>(nb) * G + cta) * kFastE;
+            if (p.k <= kFastMaxK)
+                write_ranked_list(buf, ms->sel_cnt[nb], p.k, dst, head);
+            else if (!p.pmerge)
+                write_cta_list(buf, ms->sel_cnt[nb], p.k, reinterpret_cast<uint32_t *>(smem + L.ring),
+                               reinterpret_cast<uint64_t *>(smem + L.ring + 1024), ms, dst, head);
+        }
     }
 
     // ---------------- early merge (one query, k <= 64) ----------------
@@ -1461,10 +1616,18 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
         unsigned char *ws = smem + L.merge;
         uint64_t *fe = reinterpret_cast<uint64_t *>(ws + SmemLayout::merge_fixed_bytes());
         for (int q = mg; q < p.nq; q += X) {
-            merge_published(p.flags, target, p.heads + static_cast<size_t>(q) * G * kFastE,
-                            p.cand + static_cast<size_t>(q) * G * p.k, G, p.k, ws, fe, ms, p.err,
-                            p.out_idx + static_cast<size_t>(q) * p.k, p.out_logits + static_cast<size_t>(q) * p.k,
-                            p.sparse != nullptr ? p.sparse + static_cast<int64_t>(q) * p.V : nullptr);
+            int32_t *oi = p.out_idx + static_cast<size_t>(q) * p.k;
+            float *ol = p.out_logits + static_cast<size_t>(q) * p.k;
+            float *sp = p.sparse != nullptr ? p.sparse + static_cast<int64_t>(q) * p.V : nullptr;
+            bool wide = false;
+            if constexpr (MM == 0) wide = p.k > kFastMaxK;
+            if (wide)
+                merge_published_wide(p.flags, target, p.heads + static_cast<size_t>(q) * G * kWideE,
+                                     p.cand + static_cast<size_t>(q) * G * p.list_keys, p.list_keys, G, p.k, ws,
+                                     fe, ms, p.err, oi, ol, sp);
+            else
+                merge_published(p.flags, target, p.heads + static_cast<size_t>(q) * G * kFastE,
+                                p.cand + static_cast<size_t>(q) * G * p.k, G, p.k, ws, fe, ms, p.err, oi, ol, sp);
             __syncthreads();
         }
         return;
