@@ -50,10 +50,15 @@ constexpr int kMaxHBytes = 64 * 1024;  // shared-memory budget for staged querie
 constexpr int kMaxSelBytes = 32 * 1024;  // ... and for the wide lists' candidate buffers
 // Scratch words of a handle: [0] completion ticket, [1] device flag word,
 // [2] chunk / tile pool counter, [4] launch epoch, [8 ..] one publication
-// word per CTA (a CTA's lists are ready once its word holds the epoch + 1).
+// word per CTA (a CTA's lists are ready once its word holds the epoch + 1),
+// then a counter per selector warp of the tensor-core kernel.
 constexpr int kEpochWord = 4;
 constexpr int kFlagWords = 8;
-constexpr int kNumWords = kFlagWords + vie::kMaxLists;
+constexpr int kCountWords = kFlagWords + vie::kMaxLists;
+constexpr int kNumWords = kCountWords + vie::kTcMaxSelWarps;
+// Words per CTA of the shared bounds' maxima (gmax): 8 queries x 8 on the
+// streaming path, 64 x 1 or 32 x 4 on the tensor-core path.
+constexpr int kBoundWords = 128;
 
 }  // namespace
 
@@ -67,6 +72,7 @@ struct vie_head {
     float *scale;       // e4m3 heads: fp32 scale per row [V]; nullptr for bf16 heads
     uint64_t *cand;     // [kMaxNB][G][VIE_K_MAX] ranking keys, then [kMaxNB][G][kWideE] heads
     uint32_t *words;    // kNumWords scratch words (see kEpochWord, kFlagWords)
+    uint64_t *gmax;     // [G * kBoundWords] maxima behind the shared bounds (tagged words)
     int64_t scratch_bytes;
     // tensor-core path (batches): hi/lo bf16 query matrix and TMA descriptors
     void *hB;             // [kTcHRows][d_pad] bf16, or e4m3 query pieces [4 NQ][d_pad]
@@ -176,28 +182,28 @@ __global__ void scatter_sparse_kernel(const int32_t *__restrict__ idx,
 // ---------------------------------------------------------------------------
 namespace {
 
-// Selector of the streaming kernel: register lists of 2 keys per lane (2), or
-// the shared-memory candidate buffers (0): for k > 64, and for k <= 64 where a
-// CTA's share of W is so short (rows x row_bytes up to kBufSelBytes, ~15 us of
-// its stream) that the register lists' insertions (k (1 + ln(rows / k)) keys
-// at ~0.14 us) would outlast it.
-constexpr int64_t kBufSelBytes = 640 * 1024;
-int pick_mm(int k, int64_t V, int G, int row_bytes) {
-    if (k > vie::kFastMaxK) return 0;
-    return (V + G - 1) / G * row_bytes <= kBufSelBytes ? 0 : 2;
-}
-
 // Keys per query of a launch's candidate buffers: for k <= 64 a size whose
 // keys one CTA ranks by counting; for wide lists a single query gets about 4k
 // (its first cut-back comes early in the stream, where it is hidden, and
 // usually stays the only one), groups the least size for k.
-int sel_cap_launch(int mm, int nb, int k) {
-    if (mm != 0) return 0;
+int sel_cap_launch(int nb, int k) {
     if (k <= vie::kFastMaxK) return vie::kSelCapFast;
     const int c = vie::sel_cap_for(k);
     if (nb != 1) return c;
     const int c4 = (4 * k + 63) & ~63;
     return c4 > kMaxSelBytes / 8 ? kMaxSelBytes / 8 : c4;
+}
+
+// Maxima each CTA of a streaming launch publishes per query for the shared
+// bound: the least number that gives 2k of them over the CTAs (a maximum of
+// more rows says more), at most 8; none if they would be fewer than k, or if
+// a CTA's whole share fits its buffer (k <= 64: ranking that at the end is
+// cheaper than looking for the bound: 11.6 against 12.4 us at 20011 x 640).
+int bound_blocks_for(int k, int64_t V, int G) {
+    if (k <= vie::kFastMaxK && V <= static_cast<int64_t>(vie::kSelCapFast) * G) return 0;
+    int b = 1;
+    while (b < 8 && b * G < 2 * k) b <<= 1;
+    return b * G >= k && b * G <= vie::kBoundMax ? b : 0;
 }
 
 // Widest query group for a row width and k: the staged queries and the wide
@@ -412,11 +418,14 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
     const size_t wbytes = static_cast<size_t>(V) * hd->d_pad * (e4m3 ? 1 : 2);
     const size_t cbytes =
         static_cast<size_t>(kMaxNB) * hd->G * (VIE_K_MAX + vie::kWideE) * sizeof(uint64_t);
-    hd->scratch_bytes = static_cast<int64_t>(cbytes + kNumWords * sizeof(uint32_t));
+    const size_t gbytes = static_cast<size_t>(hd->G) * kBoundWords * sizeof(uint64_t);
+    hd->scratch_bytes = static_cast<int64_t>(cbytes + gbytes + kNumWords * sizeof(uint32_t));
     e = cudaMalloc(&hd->W, wbytes);
     if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->scale, static_cast<size_t>(V) * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&hd->cand, cbytes);
     if (e == cudaSuccess) e = cudaMemset(hd->cand, 0, cbytes);  // empty lists until written
+    if (e == cudaSuccess) e = cudaMalloc(&hd->gmax, gbytes);
+    if (e == cudaSuccess) e = cudaMemset(hd->gmax, 0, gbytes);  // tag 0: of no launch
     if (e == cudaSuccess) e = cudaMalloc(&hd->words, kNumWords * sizeof(uint32_t));
     if (e == cudaSuccess)
         e = cudaMalloc(&hd->hB, static_cast<size_t>(vie::kTcHRows) * hd->d_pad * 2);
@@ -444,6 +453,7 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
         cudaFree(hd->W);
         cudaFree(hd->scale);
         cudaFree(hd->cand);
+        cudaFree(hd->gmax);
         cudaFree(hd->words);
         cudaFree(hd->hB);
         cudaFree(hd->qscale);
@@ -501,6 +511,7 @@ vie_status vie_head_destroy(vie_head *head) {
     cudaFree(head->W);
     cudaFree(head->scale);
     cudaFree(head->cand);
+    cudaFree(head->gmax);
     cudaFree(head->words);
     cudaFree(head->hB);
     cudaFree(head->qscale);
@@ -617,6 +628,11 @@ static vie_status run_topk_tc(const char *fn, vie_head *head, const float *h, in
         p.err = head->words + 1;
         p.epoch = head->words + kEpochWord;
         p.flags = head->words + kFlagWords;
+        p.counts = head->words + kCountWords;
+        p.gmax = head->gmax;
+        // a maximum per tile, or per 32 rows where the CTAs' maxima would be too few for k
+        p.gt_blocks = 2 * k <= head->G ? 1 : 4;
+        if (p.gt_blocks * head->G < k || p.gt_blocks * head->G > vie::kBoundMax) p.gt_blocks = 0;
         p.out_idx = out_idx + static_cast<int64_t>(q0) * k;
         p.out_logits = out_logits + static_cast<int64_t>(q0) * k;
         p.sparse = sparse != nullptr ? sparse + static_cast<int64_t>(q0) * head->V : nullptr;
@@ -651,17 +667,16 @@ static vie_status run_topk(const char *fn, vie_head *head, const float *h, int32
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (use_tc(head, batch, k)) return run_topk_tc(fn, head, h, batch, k, out_idx, out_logits, sparse, s);
     const int row_bytes = head->d_pad * (head->scale != nullptr ? 1 : 2);
-    const int mm = pick_mm(k, head->V, head->G, row_bytes);
     // published wide lists: the merge stages kWideE keys of every list
     const bool wide = k > vie::kFastMaxK && head->G <= vie::kThreads;
-    const uint32_t wide_bytes = vie::SmemLayout::merge_fixed_bytes() + 8u * vie::kWideE * head->G;
+    const uint32_t wide_bytes = vie::SmemLayout::merge_fixed_bytes() + 8u * (vie::kWideE + 1) * head->G;
     const int cap = nb_cap_for(head->d_pad, k);
     for (int q0 = 0; q0 < batch; q0 += cap) {
         const int nq = batch - q0 < cap ? batch - q0 : cap;
         int nb = 1;
         while (nb < nq) nb <<= 1;
         LaunchShape shp;
-        const int sel_cap = sel_cap_launch(mm, nb, k);
+        const int sel_cap = sel_cap_launch(nb, k);
         if (!pick_shape(nb, head->d_pad, row_bytes, sel_cap, wide ? wide_bytes : 0u, &shp))
             return fail(VIE_ERR_UNSUPPORTED, "%s: no shared-memory layout for d=%d", fn, head->d);
         vie::StreamTopkParams p;
@@ -698,12 +713,15 @@ static vie_status run_topk(const char *fn, vie_head *head, const float *h, int32
         // several queries, or wide lists: the first CTAs to finish merge them in parallel
         p.pmerge = (wide || (nq > 1 && k <= vie::kFastMaxK && head->G <= vie::kThreads &&
                              shp.smem - L.merge >= early_bytes)) ? 1 : 0;
+        p.gt_blocks = (p.early || p.pmerge) ? bound_blocks_for(k, head->V, head->G) : 0;
+        p.gt_tag = 0;
+        p.gmax = head->gmax;
         p.epoch = head->words + kEpochWord;
         p.flags = head->words + kFlagWords;
         p.out_idx = out_idx + static_cast<int64_t>(q0) * k;
         p.out_logits = out_logits + static_cast<int64_t>(q0) * k;
         p.sparse = sparse != nullptr ? sparse + static_cast<int64_t>(q0) * head->V : nullptr;
-        const cudaError_t e = vie::launch_stream_topk(nb, mm, shp.r, p, head->G, shp.smem, s);
+        const cudaError_t e = vie::launch_stream_topk(nb, shp.r, p, head->G, shp.smem, s);
         if (e != cudaSuccess) return fail_cuda(e, fn);
     }
     return VIE_OK;
@@ -958,6 +976,8 @@ vie_status vie_head_device_status(vie_head *head, vie_stream stream) {
     if (e != cudaSuccess) return fail_cuda(e, "vie_head_device_status: read flag");
     if (words[1] != 0) {
         e = cudaMemset(head->words, 0, 4 * sizeof(uint32_t));
+        if (e == cudaSuccess)
+            e = cudaMemset(head->words + kCountWords, 0, vie::kTcMaxSelWarps * sizeof(uint32_t));
         if (e != cudaSuccess) return fail_cuda(e, "vie_head_device_status: clear flag");
         return fail(VIE_ERR_DEVICE, "handle device flag 0x%x:%s%s", words[1],
                     (words[1] & vie::kErrWaitTimeout) ? " pipeline wait timed out" : "",
@@ -976,10 +996,11 @@ namespace {
 
 constexpr size_t kNoAllocScratchBytes = size_t(1) << 20;  // 1 MiB per device
 constexpr size_t kNoAllocCounterBytes = 256;              // counters, then the lists
+constexpr size_t kNoAllocBoundBytes = size_t(kMaxNB) * vie::kBoundMax * sizeof(uint64_t);  // behind them
 
 // Host code sees only a stand-in for this array; kernels get its device
 // address, looked up once per device below.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes + kNoAllocBoundBytes];
 
 struct NoAllocDevice {
     std::once_flag once;
@@ -1043,7 +1064,6 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
     if (g > nd.sms) g = nd.sms;
     if (g > vie::kMaxLists) g = vie::kMaxLists;
     const int G = static_cast<int>(g < 1 ? 1 : g);
-    const int mm = pick_mm(k, V, G, d * 2);
     const int cap = nb_cap_for(d, k);
     int nb_max = 1;
     while (nb_max < cap && nb_max < batch) nb_max <<= 1;
@@ -1068,13 +1088,19 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint32_t *counters = reinterpret_cast<uint32_t *>(nd.scratch);
     e = cudaMemsetAsync(counters, 0, 4 * sizeof(uint32_t), s);  // ticket and pool start at 0
+    // the shared bounds' words: none left of another call, whose tags (the
+    // group's number) repeat
+    uint64_t *gmax = reinterpret_cast<uint64_t *>(nd.scratch + kNoAllocScratchBytes);
+    const int gt_blocks = bound_blocks_for(k, V, G);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(gmax, 0, static_cast<size_t>(nb_max) * G * gt_blocks * sizeof(uint64_t), s);
     if (e != cudaSuccess) return fail_cuda(e, "vie_head_topk_noalloc clear");
     for (int q0 = 0; q0 < batch; q0 += cap) {
         const int nq = batch - q0 < cap ? batch - q0 : cap;
         int nb = 1;
         while (nb < nq) nb <<= 1;
         LaunchShape shp;
-        if (!pick_shape(nb, d, d * 2, sel_cap_launch(mm, nb, k), 0u, &shp))
+        if (!pick_shape(nb, d, d * 2, sel_cap_launch(nb, k), 0u, &shp))
             return fail(VIE_ERR_UNSUPPORTED, "%s: no shared-memory layout for d=%d", fn, d);
         vie::StreamTopkParams p;
         p.W = static_cast<const uint16_t *>(W_out);
@@ -1092,7 +1118,7 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
         p.static_chunks = static_cast<int32_t>(n_chunks * pct / 100 / G);
         p.pool_rows = pool_rows_for(shp.rs);
         p.half_rows = half_rows_for(shp.r, d / 8);
-        p.sel_cap = sel_cap_launch(mm, nb, k);
+        p.sel_cap = sel_cap_launch(nb, k);
         p.list_keys = k;
         p.cand = cand;
         p.heads = heads;
@@ -1102,34 +1128,37 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
         p.pdl = 0;    // the caller's W may come from the kernel before this one
         p.early = 0;  // the last-ticket merge: no per-CTA words in the fixed array
         p.pmerge = 0;
+        p.gt_blocks = gt_blocks;
+        p.gt_tag = static_cast<uint32_t>(q0 / cap) + 1u;
+        p.gmax = gmax;
         p.epoch = nullptr;
         p.flags = nullptr;
         p.out_idx = out_idx + static_cast<int64_t>(q0) * k;
         p.out_logits = out_logits + static_cast<int64_t>(q0) * k;
         p.sparse = nullptr;
-        e = vie::launch_stream_topk(nb, mm, shp.r, p, G, shp.smem, s);
+        e = vie::launch_stream_topk(nb, shp.r, p, G, shp.smem, s);
         if (e != cudaSuccess) return fail_cuda(e, fn);
     }
     return VIE_OK;
 }
 
 namespace vie {
-cudaError_t launch_stream_topk(int nb, int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk(int nb, int r, const StreamTopkParams &p, int grid,
                                uint32_t smem, cudaStream_t stream) {
     if (p.row_scale != nullptr) {
         switch (nb) {
-            case 1: return launch_stream_topk_e4m3_nb1(mm, r, p, grid, smem, stream);
-            case 2: return launch_stream_topk_e4m3_nb2(mm, r, p, grid, smem, stream);
-            case 4: return launch_stream_topk_e4m3_nb4(mm, r, p, grid, smem, stream);
-            case 8: return launch_stream_topk_e4m3_nb8(mm, r, p, grid, smem, stream);
+            case 1: return launch_stream_topk_e4m3_nb1(r, p, grid, smem, stream);
+            case 2: return launch_stream_topk_e4m3_nb2(r, p, grid, smem, stream);
+            case 4: return launch_stream_topk_e4m3_nb4(r, p, grid, smem, stream);
+            case 8: return launch_stream_topk_e4m3_nb8(r, p, grid, smem, stream);
             default: return cudaErrorInvalidValue;
         }
     }
     switch (nb) {
-        case 1: return launch_stream_topk_nb1(mm, r, p, grid, smem, stream);
-        case 2: return launch_stream_topk_nb2(mm, r, p, grid, smem, stream);
-        case 4: return launch_stream_topk_nb4(mm, r, p, grid, smem, stream);
-        case 8: return launch_stream_topk_nb8(mm, r, p, grid, smem, stream);
+        case 1: return launch_stream_topk_nb1(r, p, grid, smem, stream);
+        case 2: return launch_stream_topk_nb2(r, p, grid, smem, stream);
+        case 4: return launch_stream_topk_nb4(r, p, grid, smem, stream);
+        case 8: return launch_stream_topk_nb8(r, p, grid, smem, stream);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -9,28 +9,28 @@
 
 namespace vie {
 
-// Launches stream_topk_kernel<nb, mm, r> on `grid` CTAs; nb in {1,2,4,8},
-// mm in {2 (register lists), 0 (candidate buffers)}, r in {1,2,4,8}.  Returns the launch error
+// Launches stream_topk_kernel<nb, r> on `grid` CTAs; nb in {1,2,4,8}, r in
+// {1,2,4,8}.  Returns the launch error
 // (cudaErrorInvalidValue for an unsupported combination).
-cudaError_t launch_stream_topk(int nb, int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk(int nb, int r, const StreamTopkParams &p, int grid,
                                uint32_t smem, cudaStream_t stream);
 
-cudaError_t launch_stream_topk_nb1(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_nb1(int r, const StreamTopkParams &p, int grid,
                                    uint32_t smem, cudaStream_t stream);
-cudaError_t launch_stream_topk_nb2(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_nb2(int r, const StreamTopkParams &p, int grid,
                                    uint32_t smem, cudaStream_t stream);
-cudaError_t launch_stream_topk_nb4(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_nb4(int r, const StreamTopkParams &p, int grid,
                                    uint32_t smem, cudaStream_t stream);
-cudaError_t launch_stream_topk_nb8(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_nb8(int r, const StreamTopkParams &p, int grid,
                                    uint32_t smem, cudaStream_t stream);
 // The same on rows of e4m3 codes with per-row scales (p.row_scale).
-cudaError_t launch_stream_topk_e4m3_nb1(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_e4m3_nb1(int r, const StreamTopkParams &p, int grid,
                                         uint32_t smem, cudaStream_t stream);
-cudaError_t launch_stream_topk_e4m3_nb2(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_e4m3_nb2(int r, const StreamTopkParams &p, int grid,
                                         uint32_t smem, cudaStream_t stream);
-cudaError_t launch_stream_topk_e4m3_nb4(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_e4m3_nb4(int r, const StreamTopkParams &p, int grid,
                                         uint32_t smem, cudaStream_t stream);
-cudaError_t launch_stream_topk_e4m3_nb8(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_e4m3_nb8(int r, const StreamTopkParams &p, int grid,
                                         uint32_t smem, cudaStream_t stream);
 
 

@@ -13,17 +13,18 @@
 //              evict-first); the chunk id travels with the stage; an id of
 //              -1 closes the stream;
 //   warps 1..NS  selectors, NS = one per query up to four (selector s takes
-//              query slots s, s + NS, ..): per query, the best keys seen so
-//              far as a sorted list spread over the warp's registers; a row
-//              enters only if it beats the current k-th key.  They never
-//              hold a weight stage.  Wide lists (k > 64): every key above
-//              the bound tau goes into a shared-memory buffer of the query
-//              (ballot and append); a full buffer is cut back to a set
-//              holding its best k by a bisection on the keys, which raises
-//              tau.  After the stream the whole CTA turns each buffer into
-//              the sorted list (radix select of the best k, then a bitonic
-//              sort: runs of 128 keys in registers, merged through shared
-//              memory);
+//              query slots s, s + NS, ..): every key above the query's bound
+//              tau goes into its shared-memory buffer (ballot and append); a
+//              full buffer is cut back to a set holding its best k by a
+//              bisection on the keys, which raises tau.  They never hold a
+//              weight stage.  The CTAs share a bound: each publishes the
+//              largest logits of its first row blocks, and the k-th largest of
+//              all of them, read a few stages later, bounds the k-th logit of
+//              the whole vocabulary, so that only about k / G keys per CTA
+//              are left.  For k <= 64 those go into a sorted list spread over
+//              the warp's registers (an insertion is ~0.14 us), which is final
+//              when the stream ends (100003 x 1000, b = 1: 39.8 -> 33.7 us at
+//              k = 50, 49.3 -> 42.5 us at k = 300);
 //   the next 8 warps  projection: warp w owns rows w, w+8, .. (at most R) of
 //              each stage and every lane a strided set of 16-byte column
 //              chunks; bf16 -> fp32 widening, fp32 FMA against h (staged in
@@ -83,8 +84,9 @@ constexpr int kFastE = 8;              // fast merge: entries read per list (eve
 constexpr int kFastMaxK = 64;          // fast merge: largest k
 constexpr int kWideE = 32;             // published wide lists: sorted keys per list in the heads area
 constexpr int kSelCapFast = 256;       // candidate buffer keys per query, k <= kFastMaxK
+constexpr int kBoundMax = 1280;        // maxima behind a shared bound, at most
+constexpr int kBoundBlocks = 4;        // row blocks of 32 a CTA's shared maxima cover, at least
 constexpr int kSelRun = 128;           // keys of one sorted run (a warp's registers)
-constexpr int kRankRunsMin = kRankCountMax;  // merge output: a bitonic sort above this many keys
 
 // Keys per query of the shared-memory candidate buffer of the wide lists
 // (k > kFastMaxK): room for k keys and as many again, so a cut-back keeps k
@@ -108,7 +110,10 @@ struct StreamTopkParams {
     int32_t static_chunks;   // chunks each CTA owns before drawing from the pool
     int32_t pool_rows;       // rows of a pool piece (<= rows_per_stage)
     int32_t half_rows;       // 1: each half-warp projects its own row (R >= 2)
-    int32_t sel_cap;         // candidate buffers: keys per query; 0 with register lists
+    int32_t sel_cap;         // candidate buffers: keys per query
+    int32_t gt_blocks;       // shared bound: maxima each CTA publishes per query (0: none)
+    uint32_t gt_tag;         // the launch's tag in gmax (0: epoch + 1)
+    uint64_t *gmax;          // [NB][G][gt_blocks]: tag << 32 | the maximum's ordered logit
     int32_t list_keys;       // keys of a list in cand: k, or more for published wide lists
     uint64_t *cand;          // [NB][G][list_keys] keys
     uint64_t *heads;         // [NB][G][kFastE] (published wide lists: kWideE): the first keys of each list
@@ -215,6 +220,57 @@ struct WarpList {
         return shfl_u64(x, p / MM);
     }
 };
+
+// The shared bound.  g holds n words (tag << 32 | ordered logit), each the
+// largest logit of rows no other word covers; words with another tag have not
+// been written by this launch.  Returns a value at most the k-th largest of
+// them (its low 12 bits dropped), so that at least k rows have a logit of at
+// least the bound; 0 while fewer than k words are there.  n_valid counts those
+// that are.  One warp; any subset of the words gives a valid bound, so nobody
+// waits for them.
+struct SharedBound {
+    uint32_t bound;
+    int n_valid;
+};
+template <int PER>
+static __device__ __noinline__ SharedBound shared_bound(const uint64_t *g, int n, uint32_t tag, int k, int lane) {
+    uint32_t v[PER];
+    int have = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const uint64_t x = j * 32 + lane < n ? ld_relaxed_gpu_u64(g + j * 32 + lane) : 0ull;
+        v[j] = static_cast<uint32_t>(x >> 32) == tag ? static_cast<uint32_t>(x) : 0u;
+        have += v[j] != 0 ? 1 : 0;
+    }
+    have = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(have)));
+    uint32_t th = 0;
+    if (have >= k) {
+#pragma unroll 1
+        for (int bit = 30; bit >= 12; bit -= 2) {
+            const uint32_t c1 = th | (1u << bit), c2 = th | (2u << bit), c3 = th | (3u << bit);
+            unsigned n1 = 0, n2 = 0, n3 = 0;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                n1 += v[j] >= c1 ? 1 : 0;
+                n2 += v[j] >= c2 ? 1 : 0;
+                n3 += v[j] >= c3 ? 1 : 0;
+            }
+            // three counts of at most kBoundMax in one reduction each
+            n1 = __reduce_add_sync(0xFFFFFFFFu, n1 | (n2 << 16));
+            n3 = __reduce_add_sync(0xFFFFFFFFu, n3);
+            n2 = n1 >> 16;
+            n1 &= 0xFFFFu;
+            const unsigned uk = static_cast<unsigned>(k);
+            th = n3 >= uk ? c3 : (n2 >= uk ? c2 : (n1 >= uk ? c1 : th));
+        }
+    }
+    return SharedBound{th, have};
+}
+__device__ __forceinline__ SharedBound shared_bound(const uint64_t *g, int n, uint32_t tag, int k, int lane) {
+    if (n <= 160) return shared_bound<5>(g, n, tag, k, lane);
+    if (n <= 640) return shared_bound<20>(g, n, tag, k, lane);
+    return shared_bound<kBoundMax / 32>(g, n, tag, k, lane);
+}
 
 // Bitonic sort, descending, of the 32 * PER keys a warp holds (lane l holds
 // elements l*PER .. l*PER + PER - 1).  Steps with a stride below PER swap
@@ -440,53 +496,6 @@ __device__ inline void block_sort_desc(uint64_t *a, int m) {
     __syncthreads();
 }
 
-// Exact top-k of n unique nonzero keys in shared memory, written best first
-// to out_idx / out_logits (and into the sparse row, if any).  Rank counting
-// for small n, otherwise a radix-select threshold and rank counting of the
-// k winners.
-__device__ inline void block_topk_to_output(uint64_t *keys, int n, int k, uint64_t *win,
-                                            uint32_t *hist, MiscSmem *ms, int32_t *out_idx,
-                                            float *out_logits, float *sparse_row) {
-    const int tid = threadIdx.x;
-    uint64_t *src = keys;
-    int m = n;
-    if (n > kRankCountMax && n > k) {
-        const uint64_t T = block_radix_threshold(SmemKeys{keys}, n, k, 1, hist, ms);
-        if (tid == 0) ms->n_win = 0;
-        __syncthreads();
-        for (int i = tid; i < n; i += static_cast<int>(blockDim.x)) {
-            const uint64_t x = keys[i];
-            if (x >= T) win[atomicAdd(&ms->n_win, 1)] = x;
-        }
-        __syncthreads();
-        src = win;
-        m = k;
-    }
-    if (m > kRankRunsMin) {
-        // many keys: a bitonic sort (rank counting is m^2); src has room for
-        // the sort's power of two (at most 1024 keys here)
-        block_sort_desc(src, m);
-        for (int i = tid; i < min(m, k); i += static_cast<int>(blockDim.x)) {
-            const uint64_t x = src[i];
-            out_idx[i] = key_index(x);
-            out_logits[i] = key_value(x);
-            if (sparse_row != nullptr) sparse_row[key_index(x)] = key_value(x);
-        }
-        __syncthreads();
-        return;
-    }
-    for (int i = tid; i < m; i += static_cast<int>(blockDim.x)) {
-        const uint64_t x = src[i];
-        const int rank = rank_among(src, m, x);
-        if (rank < k) {
-            out_idx[rank] = key_index(x);
-            out_logits[rank] = key_value(x);
-            if (sparse_row != nullptr) sparse_row[key_index(x)] = key_value(x);
-        }
-    }
-    __syncthreads();
-}
-
 // Wide lists: cuts the cnt (> k) unique nonzero keys of buf back to a set
 // that holds its best k, moved to buf[0..), and returns its size and the new
 // entry bound (a later key enters only if it is above the bound).
@@ -619,10 +628,25 @@ __device__ inline void write_cta_list(uint64_t *buf, int cnt, int k, uint32_t *h
     for (int i = m + tid; i < kFastE; i += nthr) head[i] = 0ull;
 }
 
-// The same for k <= kFastMaxK: every key of the buffer (at most kSelCapFast)
-// is ranked by counting the keys above it, one thread per key, and the best k
-// go out at their rank.  About 0.5 us for 256 keys, where a sorted register
-// list pays ~0.14 us for every key that enters it.
+// The cnt unique nonzero keys of buf above tau, moved to buf[0..) in order;
+// returns how many.  One warp.
+static __device__ __noinline__ int warp_filter(uint64_t *buf, int cnt, uint64_t tau, int lane) {
+    __syncwarp();
+    const unsigned lt_mask = (1u << lane) - 1u;
+    int base = 0;
+    for (int e0 = 0; e0 < cnt; e0 += 32) {  // in place, as in warp_cut_back
+        const uint64_t v = e0 + lane < cnt ? buf[e0 + lane] : 0ull;
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, v > tau);
+        if (v > tau) buf[base + __popc(m & lt_mask)] = v;
+        base += __popc(m);
+    }
+    __syncwarp();
+    return base;
+}
+
+// The same for k <= kFastMaxK (streams too short for the shared bound): every key of the buffer (at most kSelCapFast) is ranked by counting the keys
+// above it, one thread per key, and the best k go out at their rank (~1.5 us
+// for 224 keys).
 __device__ inline void write_ranked_list(const uint64_t *buf, int cnt, int k, uint64_t *dst, uint64_t *head) {
     const int tid = threadIdx.x, nthr = static_cast<int>(blockDim.x);
     for (int i = tid; i < cnt; i += nthr) {
@@ -664,6 +688,115 @@ struct MergeBufs {
     int *counts, *offsets;
     uint32_t *hist;
 };
+
+// Exact top-k of n (at most kMergeCandCap) unique nonzero keys in shared
+// memory (not mb.pref), written best first to out_idx / out_logits (and into
+// the sparse row, if any).  A counting sort by logit: the keys' range of
+// ordered logits is cut into kRankBins equal bins, a key's rank is the number
+// of keys in higher bins plus the number above it in its own.  Every thread of
+// the CTA (at least kThreads) calls it.  (Ranking by comparing all pairs takes
+// ~3.7 us for 440 keys; where ties or outliers crowd more than kRankCrowd keys
+// into one bin, the keys are sorted instead.)
+constexpr int kRankBins = 512;
+constexpr int kRankCrowd = 160;
+__device__ inline void block_topk_to_output(const uint64_t *keys, int n, int k, const MergeBufs &mb, MiscSmem *ms,
+                                            int32_t *out_idx, float *out_logits, float *sparse_row) {
+    constexpr int PER = (kMergeCandCap + kThreads - 1) / kThreads;  // keys per thread
+    static_assert(kRankBins <= kMaxLists && kMergeCandCap <= kMergePrefixCap, "bins and keys fit their buffers");
+    const int tid = threadIdx.x, lane = tid & 31, nthr = static_cast<int>(blockDim.x);
+    int *bin = mb.counts, *above = mb.offsets;  // keys of a bin, keys of all higher bins
+    uint32_t *range = mb.hist;                  // [0] lowest, [1] highest ordered logit
+    uint64_t *sorted = mb.pref;                 // the keys by bin, highest first
+    for (int i = tid; i < kRankBins; i += nthr) bin[i] = 0;
+    if (tid == 0) {
+        range[0] = 0xFFFFFFFFu;
+        range[1] = 0u;
+        range[2] = 0u;  // 1: a crowded bin
+    }
+    __syncthreads();
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+    for (int i = tid; i < n; i += nthr) {
+        const uint32_t v = static_cast<uint32_t>(keys[i] >> 32);
+        lo = min(lo, v);
+        hi = max(hi, v);
+    }
+    lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+    hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+    if (lane == 0) {
+        atomicMin(&range[0], lo);
+        atomicMax(&range[1], hi);
+    }
+    __syncthreads();
+    lo = range[0];
+    const uint32_t span = range[1] - lo;
+    const int bits = 32 - __clz(static_cast<int>(span));
+    const int shift = n > 0 && bits > 9 ? bits - 9 : 0;
+    static_assert(kRankBins == 1 << 9, "bins cover the range");
+    int pos[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = tid + j * nthr;
+        if (i < n) pos[j] = atomicAdd(&bin[(static_cast<uint32_t>(keys[i] >> 32) - lo) >> shift], 1);
+    }
+    __syncthreads();
+    if (tid < 32) {  // lane l: the bins kRankBins - 1 - 16 l, downwards
+        constexpr int BL = kRankBins / 32;
+        int c[BL], local = 0;
+#pragma unroll
+        for (int j = 0; j < BL; ++j) {
+            c[j] = bin[kRankBins - 1 - BL * lane - j];
+            local += c[j];
+        }
+        int incl = local;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        int run = incl - local;
+#pragma unroll
+        for (int j = 0; j < BL; ++j) {
+            above[kRankBins - 1 - BL * lane - j] = run;
+            run += c[j];
+            if (c[j] > kRankCrowd) range[2] = 1u;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = tid + j * nthr;
+        if (i < n) {
+            const uint64_t x = keys[i];
+            sorted[above[(static_cast<uint32_t>(x >> 32) - lo) >> shift] + pos[j]] = x;
+        }
+    }
+    __syncthreads();
+    if (range[2] != 0) {
+        block_sort_desc(sorted, n);  // (n <= 2048 keys: the power of two above fits)
+        for (int i = tid; i < min(n, k); i += nthr) {
+            const uint64_t x = sorted[i];
+            out_idx[i] = key_index(x);
+            out_logits[i] = key_value(x);
+            if (sparse_row != nullptr) sparse_row[key_index(x)] = key_value(x);
+        }
+        __syncthreads();
+        return;
+    }
+    for (int i = tid; i < n; i += nthr) {
+        const uint64_t x = sorted[i];
+        const int b = static_cast<int>((static_cast<uint32_t>(x >> 32) - lo) >> shift);
+        const int first = above[b], last = first + bin[b];
+        if (first >= k) continue;
+        int rank = first;
+        for (int j = first; j < last; ++j) rank += sorted[j] > x ? 1 : 0;
+        if (rank < k) {
+            out_idx[rank] = key_index(x);
+            out_logits[rank] = key_value(x);
+            if (sparse_row != nullptr) sparse_row[key_index(x)] = key_value(x);
+        }
+    }
+    __syncthreads();
+}
 
 // Merges the G sorted lists of one query (G x k keys, `lists`) into the
 // exact top-k.  Keys = SmemKeys when the lists were staged in shared memory.
@@ -746,7 +879,7 @@ __device__ void merge_lists(Keys lists, int G, int k, const MergeBufs &mb, MiscS
                 mb.cands[mb.offsets[c] + j] =
                     (have_pref && j < J) ? mb.pref[c * J + j] : lists[c * k + j];
         __syncthreads();
-        block_topk_to_output(mb.cands, M, k, mb.win, mb.hist, ms, oi, ol, sp);
+        block_topk_to_output(mb.cands, M, k, mb, ms, oi, ol, sp);
     } else {
         // 3b. too many candidates: radix-select the threshold over all lists
         const uint64_t T = block_radix_threshold(lists, G * k, k, lo, mb.hist, ms);
@@ -757,7 +890,7 @@ __device__ void merge_lists(Keys lists, int G, int k, const MergeBufs &mb, MiscS
             if (x >= T && x >= lo) mb.win[atomicAdd(&ms->n_win, 1)] = x;
         }
         __syncthreads();
-        block_topk_to_output(mb.win, k, k, mb.win, mb.hist, ms, oi, ol, sp);
+        block_topk_to_output(mb.win, k, k, mb, ms, oi, ol, sp);
     }
 }
 
@@ -778,9 +911,9 @@ __device__ __forceinline__ void merge_fast_reset(int *rank_part, MiscSmem *ms) {
 // their heads' value bits (padded with 0 to a multiple of 8).  tau = the
 // k-th largest head value counted with multiplicity: at least k keys are
 // >= (tau << 32), so every top-k key is too, and each list contributes its
-// prefix of keys above that bound.  Returns false (writing nothing) if some
-// list might hold more than kFastE such keys or fewer than k heads are
-// real; the caller then merges in full.  Requires 2 * G <= kThreads, and
+// prefix of keys above that bound (all its keys when fewer than k heads are
+// real).  Returns false (writing nothing) if some list might hold more than
+// kFastE such keys; the caller then merges in full.  Requires 2 * G <= kThreads, and
 // the state merge_fast_reset sets, made visible by a bar.sync.
 __device__ inline bool merge_fast_query(const uint64_t *fe, const uint32_t *hv, int G, int k,
                                         uint64_t *cands, int *rank_part, MiscSmem *ms, int32_t *oi,
@@ -805,9 +938,10 @@ __device__ inline bool merge_fast_query(const uint64_t *fe, const uint32_t *hv, 
         if (lane == 0 && best != 0) atomicMax(&ms->tau_v, best);
     }
     __syncthreads();
+    // fewer than k real heads (lists cut to a shared bound are mostly empty):
+    // every key of every list is a candidate
     const uint32_t tv = ms->tau_v;
-    if (tv == 0) return false;  // uniform: fewer than k real heads
-    const uint64_t lo = static_cast<uint64_t>(tv) << 32;
+    const uint64_t lo = tv == 0 ? 1ull : static_cast<uint64_t>(tv) << 32;
     const int En = k < kFastE ? k : kFastE;
     // gather: list c's keys >= lo, slots taken per warp
     {
@@ -1021,14 +1155,17 @@ __device__ inline void merge_published(const uint32_t *flags, uint32_t target, c
 // Merge of one query from published wide lists (k > kFastMaxK; every thread
 // of the merging CTA, at least G threads): polls the publication words as
 // merge_published does, then
-//   1. brings the lists' heads (G x kWideE sorted keys) into shared memory;
+//   1. gathers the lists' heads (up to kWideE keys each; lists cut to the
+//      shared bound hold little more than k keys in all): if no head is full
+//      and they fit the candidate buffer, the exact top-k of them is the
+//      answer; otherwise
 //   2. tau = the k-th largest key among the first J of every list (a lower
 //      bound on the k-th key, 0 if they hold fewer than k keys);
 //   3. unless some list's last head key is still >= tau (it may hold more),
 //      the exact top-k of the head keys >= tau is the answer; otherwise every
 //      key >= tau is gathered from the whole lists (lists_q, G x list_keys,
 //      unsorted, zeros as empty slots).
-// ws holds the merge buffers (merge_fixed_bytes), fe G * kWideE keys.
+// ws holds the merge buffers (merge_fixed_bytes), fe G * (kWideE + 1) keys.
 __device__ inline void merge_published_wide(const uint32_t *flags, uint32_t target, const uint64_t *heads_q,
                                             const uint64_t *lists_q, int list_keys, int G, int k,
                                             unsigned char *ws, uint64_t *fe, MiscSmem *ms, uint32_t *err,
@@ -1059,20 +1196,47 @@ __device__ inline void merge_published_wide(const uint32_t *flags, uint32_t targ
         }
         if (__syncthreads_count(pending ? 1 : 0) == 0) break;
     }
-    // 1. the heads
+    // 1. the heads, staged with one key of padding per list (thread c then
+    // walks list c without bank conflicts)
     const int n_heads = G * kWideE;
     const ulonglong2 *src2 = reinterpret_cast<const ulonglong2 *>(heads_q);
-    ulonglong2 *fe2 = reinterpret_cast<ulonglong2 *>(fe);
-#pragma unroll 4
-    for (int i = tid; i < n_heads / 2; i += nthr) fe2[i] = __ldcg(src2 + i);
+#pragma unroll 8
+    for (int i = tid; i < n_heads / 2; i += nthr) {
+        const ulonglong2 x = __ldcg(src2 + i);
+        uint64_t *f = fe + 2 * i + 2 * i / kWideE;
+        f[0] = x.x;
+        f[1] = x.y;
+    }
     __syncthreads();
+    {
+        const uint64_t *f = fe + tid * (kWideE + 1);
+        int n = 0;
+        if (tid < G)
+            while (n < kWideE && f[n] != 0) ++n;
+        if (n == kWideE) ms->overflow = 1;  // the list may hold more
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        int base = 0;
+        if (lane == 31 && incl > 0) base = atomicAdd(&ms->n_cand, incl);
+        base = __shfl_sync(0xFFFFFFFFu, base, 31) + incl - n;
+        for (int j = 0; j < n && base + j < kMergeCandCap; ++j) mb.cands[base + j] = f[j];
+    }
+    __syncthreads();
+    if (!ms->overflow && ms->n_cand <= kMergeCandCap) {  // every key there is
+        block_topk_to_output(mb.cands, ms->n_cand, k, mb, ms, oi, ol, sp);
+        return;
+    }
     // 2. tau from the first J keys of every list: twice the expected share
     int J = (2 * k + G - 1) / G;
     J = min(J, min(kWideE, kMergePrefixCap / G));
     const int P = G * J;
     int nz = 0;
     for (int i = tid; i < P; i += nthr) {
-        const uint64_t x = fe[(i / J) * kWideE + i % J];
+        const uint64_t x = fe[(i / J) * (kWideE + 1) + i % J];
         mb.pref[i] = x;
         nz += x != 0 ? 1 : 0;
     }
@@ -1080,14 +1244,21 @@ __device__ inline void merge_published_wide(const uint32_t *flags, uint32_t targ
     if (lane == 0 && nz != 0) atomicAdd(&ms->remaining, nz);
     __syncthreads();
     const bool enough = ms->remaining >= k;
-    __syncthreads();  // block_radix_threshold reuses the word
+    if (tid == 0) {
+        ms->n_cand = 0;
+        ms->overflow = 0;
+    }
+    __syncthreads();  // block_radix_threshold reuses `remaining`
     const uint64_t tau = enough ? block_radix_threshold(SmemKeys{mb.pref}, P, k, 1, mb.hist, ms) : 0;
     const uint64_t lo = tau > 0 ? tau : 1;
-    // 3. the candidates
-    if (tid < G && fe[tid * kWideE + kWideE - 1] >= lo) ms->overflow = 1;
+    // 3. the keys >= tau
+    if (tid < G && fe[tid * (kWideE + 1) + kWideE - 1] >= lo) ms->overflow = 1;
     __syncthreads();
     const bool whole = ms->overflow != 0;
-    const int n = whole ? G * list_keys : n_heads;
+    const int n_staged = G * (kWideE + 1);  // (the padding is zeroed below)
+    if (tid < G) fe[tid * (kWideE + 1) + kWideE] = 0ull;
+    __syncthreads();
+    const int n = whole ? G * list_keys : n_staged;
     for (int i0 = tid - lane; i0 < n; i0 += nthr) {
         const int i = i0 + lane;
         uint64_t x = 0;
@@ -1103,7 +1274,7 @@ __device__ inline void merge_published_wide(const uint32_t *flags, uint32_t targ
     __syncthreads();
     const int M = ms->n_cand;
     if (M <= kMergeCandCap) {
-        block_topk_to_output(mb.cands, M, k, mb.win, mb.hist, ms, oi, ol, sp);
+        block_topk_to_output(mb.cands, M, k, mb, ms, oi, ol, sp);
         return;
     }
     // too many for the buffer: the exact threshold first
@@ -1114,7 +1285,7 @@ __device__ inline void merge_published_wide(const uint32_t *flags, uint32_t targ
         if (x >= T && x >= lo) mb.win[atomicAdd(&ms->n_win, 1)] = x;
     }
     __syncthreads();
-    block_topk_to_output(mb.win, k, k, mb.win, mb.hist, ms, oi, ol, sp);
+    block_topk_to_output(mb.win, k, k, mb, ms, oi, ol, sp);
 }
 
 // --------------------------------------------------------------------------
@@ -1151,7 +1322,7 @@ __device__ __forceinline__ float fma_e4m3x4(uint32_t w, float4 h, float a) {
 //
 // Q8: rows of e4m3 codes (16 per 16-byte chunk) with one fp32 scale per row,
 // logit = scale * sum; otherwise bf16 rows (8 per chunk).
-template <int NB, int MM, int R, bool Q8>
+template <int NB, int R, bool Q8>
 __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const StreamTopkParams p) {
     constexpr int NS = sel_warps<NB>(), T = threads_for<NB>(), QPS = NB / NS;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -1159,7 +1330,7 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
     const int S = p.stages;
     const int row_bytes = Q8 ? p.d_pad : p.d_pad * 2;
     constexpr int kEPC = Q8 ? 16 : 8;  // weights per 16-byte chunk
-    const SmemLayout L(NB, p.d_pad, RS, S, row_bytes, MM == 0 ? p.sel_cap : 0);
+    const SmemLayout L(NB, p.d_pad, RS, S, row_bytes, p.sel_cap);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + L.bars);
     uint64_t *empty = full + kMaxStages;
     uint64_t *sfull = empty + kMaxStages;
@@ -1283,128 +1454,142 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
         named_barrier_sync(1, T - 32);  // h in shared memory for warps 1..
         if (warp <= NS) {
             const int sw = NS == 1 ? 0 : warp - 1;  // this selector's query slots: sw, sw + NS, ...
-            if constexpr (MM == 0) {
-                // ---------------- selector (wide lists) ----------------
-                uint64_t *sbuf = reinterpret_cast<uint64_t *>(smem + L.sel);
-                const int cap = p.sel_cap;
-                const unsigned lt_mask = (1u << lane) - 1u;
-                int cnt[QPS];
-                uint64_t tau[QPS];
+            // ---------------- selector ----------------
+            uint64_t *sbuf = reinterpret_cast<uint64_t *>(smem + L.sel);
+            const int cap = p.sel_cap;
+            const unsigned lt_mask = (1u << lane) - 1u;
+            int cnt[QPS];
+            uint64_t tau[QPS];
+            // the shared bound: the first n_smp row blocks give gt_blocks
+            // maxima of `span` blocks each
+            const int span = max(1, kBoundBlocks / max(1, p.gt_blocks));
+            const int n_smp = p.gt_blocks * span, n_max = G * p.gt_blocks;
+            const uint32_t tag = p.gt_tag != 0 ? p.gt_tag : ms->epoch + 1u;
+            uint32_t mx[QPS];
+            WarpList<2> list[QPS];       // k <= kFastMaxK, once bounded: the keys so far, sorted
+            bool listed[QPS];
+            int blk = 0;                 // row blocks seen
+            bool bounded = n_smp == 0;   // the bound over all CTAs has been taken
+            int next_look = 0x7FFFFFFF;  // stage at which it is looked for
+            auto look = [&]() {
+                bounded = true;
 #pragma unroll
                 for (int j = 0; j < QPS; ++j) {
-                    cnt[j] = 0;
-                    tau[j] = 0;
-                }
-                for (int t = 0;; ++t) {
-                    const int s = t % kScoreStages, u = t / kScoreStages;
-                    if (!mbar_wait(&sfull[s], u & 1, abort_flag)) {
-                        if (lane == 0) {
-                            atomicOr(p.err, kErrWaitTimeout);
-                            ms->abort = 1;
-                        }
-                        break;
+                    const int nb = sw + j * NS;
+                    if (nb >= p.nq) break;
+                    const SharedBound sb =
+                        shared_bound(p.gmax + static_cast<size_t>(nb) * n_max, n_max, tag, p.k, lane);
+                    if (sb.bound != 0) tau[j] = max(tau[j], (static_cast<uint64_t>(sb.bound) << 32) - 1u);
+                    bounded = bounded && sb.n_valid == n_max;
+                    uint64_t *buf = sbuf + nb * cap;
+                    cnt[j] = warp_filter(buf, cnt[j], tau[j], lane);
+                    if (p.k <= kFastMaxK && !listed[j] && cnt[j] <= 32) {
+                        for (int i = 0; i < cnt[j]; ++i) list[j].insert(buf[i], lane);
+                        tau[j] = max(tau[j], list[j].at(p.k - 1));
+                        listed[j] = true;
                     }
-                    const int chunk = ms->chunk_s[s];
-                    if (chunk < 0) break;
-                    const int64_t row0 = chunk;
-                    const int rows = stage_rows(row0, pool_row0, RS, RSH, p.V);
-                    const float *sc = scores + s * RS * NB;
+                }
+            };
 #pragma unroll
-                    for (int j = 0; j < QPS; ++j) {
-                        const int nb = sw + j * NS;
-                        if (nb >= p.nq) break;
-                        uint64_t *buf = sbuf + nb * cap;
-                        for (int rb = 0; rb < rows; rb += 32) {
-                            if (cnt[j] > cap - 32) {  // no room for another 32 keys: cut back
+            for (int j = 0; j < QPS; ++j) {
+                cnt[j] = 0;
+                tau[j] = 0;
+                mx[j] = 0;
+                list[j].clear();
+                listed[j] = false;
+            }
+            for (int t = 0;; ++t) {
+                const int s = t % kScoreStages, u = t / kScoreStages;
+                if (!mbar_wait(&sfull[s], u & 1, abort_flag)) {
+                    if (lane == 0) {
+                        atomicOr(p.err, kErrWaitTimeout);
+                        ms->abort = 1;
+                    }
+                    break;
+                }
+                const int chunk = ms->chunk_s[s];
+                if (chunk < 0) break;
+                const int64_t row0 = chunk;
+                const int rows = stage_rows(row0, pool_row0, RS, RSH, p.V);
+                const float *sc = scores + s * RS * NB;
+                if (!bounded && t >= next_look) {
+                    look();
+                    next_look = t + 4;
+                }
+#pragma unroll
+                for (int j = 0; j < QPS; ++j) {
+                    const int nb = sw + j * NS;
+                    if (nb >= p.nq) break;
+                    uint64_t *buf = sbuf + nb * cap;
+                    for (int rb = 0; rb < rows; rb += 32) {
+                        if (cnt[j] > cap - 32) {  // no room (never once listed) for another 32 keys: cut back
+                            cnt[j] = warp_filter(buf, cnt[j], tau[j], lane);
+                            if (cnt[j] > (cap + p.k) / 2) {
                                 const CutBack cb = warp_cut_back(buf, cnt[j], p.k, (cap + p.k) / 2, lane);
                                 cnt[j] = cb.n;
                                 tau[j] = cb.bound;
                             }
-                            const int r = rb + lane;
-                            const uint64_t key =
-                                (r < rows) ? make_key(sc[r * NB + nb], static_cast<uint32_t>(row0 + r)) : 0;
-                            const bool in = key > tau[j];
-                            const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
+                        }
+                        const int r = rb + lane;
+                        const uint64_t key =
+                            (r < rows) ? make_key(sc[r * NB + nb], static_cast<uint32_t>(row0 + r)) : 0;
+                        const int b = blk + (rb >> 5);
+                        if (b < n_smp) {
+                            mx[j] = max(mx[j], __reduce_max_sync(0xFFFFFFFFu, static_cast<uint32_t>(key >> 32)));
+                            if ((b & (span - 1)) == span - 1) {
+                                if (lane == 0)
+                                    st_relaxed_gpu_u64(p.gmax + (static_cast<size_t>(nb) * G + cta) * p.gt_blocks + b / span,
+                                                       (static_cast<uint64_t>(tag) << 32) | mx[j]);
+                                mx[j] = 0;
+                            }
+                        }
+                        const bool in = key > tau[j];
+                        unsigned m = __ballot_sync(0xFFFFFFFFu, in);
+                        if (listed[j]) {
+                            if (m) {
+                                do {
+                                    const int src = __ffs(m) - 1;
+                                    m &= m - 1;
+                                    list[j].insert(shfl_u64(key, src), lane);
+                                } while (m);
+                                tau[j] = max(tau[j], list[j].at(p.k - 1));
+                            }
+                        } else {
                             if (in) buf[cnt[j] + __popc(m & lt_mask)] = key;
                             cnt[j] += __popc(m);
                         }
                     }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sempty[s]);
                 }
-                if (p.k > kFastMaxK && p.pmerge) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sempty[s]);
+                if (blk < n_smp && blk + ((rows + 31) >> 5) >= n_smp) next_look = t + 3;
+                blk += (rows + 31) >> 5;
+            }
+            // the lists -> scratch: by this warp, or (sel_cnt: no bound yet, as
+            // on short streams, or wide lists that are not published) by the
+            // whole CTA below
+            if (!bounded && p.k > kFastMaxK) look();
 #pragma unroll
-                    for (int j = 0; j < QPS; ++j) {
-                        const int nb = sw + j * NS;
-                        if (nb < p.nq)
-                            write_wide_list(sbuf + nb * cap, cnt[j], p.k, p.list_keys,
-                                            p.cand + (static_cast<size_t>(nb) * G + cta) * p.list_keys,
-                                            p.heads + (static_cast<size_t>(nb) * G + cta) * kWideE, lane);
-                    }
-                } else if (lane == 0) {
-#pragma unroll
-                    for (int j = 0; j < QPS; ++j) ms->sel_cnt[sw + j * NS] = sw + j * NS < p.nq ? cnt[j] : 0;
-                }
-            } else {
-                // ---------------- selector ----------------
-                WarpList<MM> list[QPS];
-                uint64_t tau[QPS];
-#pragma unroll
-                for (int j = 0; j < QPS; ++j) {
-                    list[j].clear();
-                    tau[j] = 0;
-                }
-                for (int t = 0;; ++t) {
-                    const int s = t % kScoreStages, u = t / kScoreStages;
-                    if (!mbar_wait(&sfull[s], u & 1, abort_flag)) {
-                        if (lane == 0) {
-                            atomicOr(p.err, kErrWaitTimeout);
-                            ms->abort = 1;
-                        }
-                        break;
-                    }
-                    const int chunk = ms->chunk_s[s];
-                    if (chunk < 0) break;
-                    const int64_t row0 = chunk;
-                    const int rows = stage_rows(row0, pool_row0, RS, RSH, p.V);
-                    const float *sc = scores + s * RS * NB;
-#pragma unroll
-                    for (int j = 0; j < QPS; ++j) {
-                        const int nb = sw + j * NS;
-                        if (nb >= p.nq) break;
-                        for (int rb = 0; rb < rows; rb += 32) {
-                            const int r = rb + lane;
-                            const uint64_t key =
-                                (r < rows) ? make_key(sc[r * NB + nb], static_cast<uint32_t>(row0 + r)) : 0;
-                            unsigned m = __ballot_sync(0xFFFFFFFFu, key > tau[j]);
-                            while (m) {
-                                const int srcl = __ffs(m) - 1;
-                                m &= m - 1;
-                                const uint64_t x = shfl_u64(key, srcl);
-                                if (x > tau[j]) {
-                                    list[j].insert(x, lane);
-                                    tau[j] = list[j].at(p.k - 1);
-                                }
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sempty[s]);
-                }
-                // this CTA's sorted top-k per query -> scratch (every slot,
-                // zeros for the unused ones)
-#pragma unroll
-                for (int j = 0; j < QPS; ++j) {
-                    const int nb = sw + j * NS;
-                    uint64_t *dst = p.cand + (static_cast<size_t>(nb) * G + cta) * p.k;
+            for (int j = 0; j < QPS; ++j) {
+                const int nb = sw + j * NS;
+                if (nb >= p.nq) break;
+                uint64_t *dst = p.cand + (static_cast<size_t>(nb) * G + cta) * p.list_keys;
+                int left = -1;
+                if (listed[j]) {
                     uint64_t *head = p.heads + (static_cast<size_t>(nb) * G + cta) * kFastE;
 #pragma unroll
-                    for (int s = 0; s < MM; ++s) {
-                        const int pos = lane * MM + s;
-                        if (pos < p.k) dst[pos] = list[j].v[s];
-                        if (pos < kFastE) head[pos] = pos < p.k ? list[j].v[s] : 0ull;
+                    for (int i = 0; i < 2; ++i) {
+                        const int pos = lane * 2 + i;
+                        if (pos < p.k) dst[pos] = list[j].v[i];
+                        if (pos < kFastE) head[pos] = pos < p.k ? list[j].v[i] : 0ull;
                     }
+                } else if (p.k > kFastMaxK && p.pmerge) {
+                    write_wide_list(sbuf + nb * cap, cnt[j], p.k, p.list_keys, dst,
+                                    p.heads + (static_cast<size_t>(nb) * G + cta) * kWideE, lane);
+                } else {
+                    left = cnt[j];
                 }
+                if (lane == 0) ms->sel_cnt[nb] = left;
             }
         } else {
             // ---------------- projection ----------------
@@ -1551,21 +1736,20 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
     }
 
     // ---------------- buffers -> sorted lists ----------------
-    // (the ring is free: every stage was consumed before its role ended;
-    // published wide lists have been written by the selectors already)
-    if constexpr (MM == 0) {
-        __syncthreads();
-        uint64_t *sbuf = reinterpret_cast<uint64_t *>(smem + L.sel);
-        for (int nb = 0; nb < p.nq; ++nb) {
-            uint64_t *buf = sbuf + nb * p.sel_cap;
-            uint64_t *dst = p.cand + (static_cast<size_t>(nb) * G + cta) * p.k;
-            uint64_t *head = p.heads + (static_cast<size_t>(nb) * G + cta) * kFastE;
-            if (p.k <= kFastMaxK)
-                write_ranked_list(buf, ms->sel_cnt[nb], p.k, dst, head);
-            else if (!p.pmerge)
-                write_cta_list(buf, ms->sel_cnt[nb], p.k, reinterpret_cast<uint32_t *>(smem + L.ring),
-                               reinterpret_cast<uint64_t *>(smem + L.ring + 1024), ms, dst, head);
-        }
+    // (those the selectors have not written; the ring is free: every stage was
+    // consumed before its role ended)
+    __syncthreads();
+    for (int nb = 0; nb < p.nq; ++nb) {
+        const int left = ms->sel_cnt[nb];
+        if (left < 0) continue;
+        uint64_t *buf = reinterpret_cast<uint64_t *>(smem + L.sel) + nb * p.sel_cap;
+        uint64_t *dst = p.cand + (static_cast<size_t>(nb) * G + cta) * p.k;
+        uint64_t *head = p.heads + (static_cast<size_t>(nb) * G + cta) * kFastE;
+        if (p.k <= kFastMaxK)
+            write_ranked_list(buf, left, p.k, dst, head);
+        else
+            write_cta_list(buf, left, p.k, reinterpret_cast<uint32_t *>(smem + L.ring),
+                           reinterpret_cast<uint64_t *>(smem + L.ring + 1024), ms, dst, head);
     }
 
     // ---------------- early merge (one query, k <= 64) ----------------
@@ -1619,9 +1803,7 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
             int32_t *oi = p.out_idx + static_cast<size_t>(q) * p.k;
             float *ol = p.out_logits + static_cast<size_t>(q) * p.k;
             float *sp = p.sparse != nullptr ? p.sparse + static_cast<int64_t>(q) * p.V : nullptr;
-            bool wide = false;
-            if constexpr (MM == 0) wide = p.k > kFastMaxK;
-            if (wide)
+            if (p.k > kFastMaxK)
                 merge_published_wide(p.flags, target, p.heads + static_cast<size_t>(q) * G * kWideE,
                                      p.cand + static_cast<size_t>(q) * G * p.list_keys, p.list_keys, G, p.k, ws,
                                      fe, ms, p.err, oi, ol, sp);

@@ -2,8 +2,8 @@
 #include "vie_stream_topk_inst.cuh"
 
 namespace vie {
-cudaError_t launch_stream_topk_e4m3_nb1(int mm, int r, const StreamTopkParams &p, int grid,
+cudaError_t launch_stream_topk_e4m3_nb1(int r, const StreamTopkParams &p, int grid,
                                         uint32_t smem, cudaStream_t stream) {
-    return launch_width<1, true>(mm, r, p, grid, smem, stream);
+    return launch_width<1, true>(r, p, grid, smem, stream);
 }
 }  // namespace vie

@@ -22,7 +22,16 @@
 //                NQ = 64): per query a sorted list of the best keys so far,
 //                spread over the warp's registers (the streaming kernel's
 //                WarpList); a row enters only when its key beats the list's
-//                k-th, so the lists are final when the stream ends.
+//                k-th, so the lists are final when the stream ends.  An
+//                insertion costs ~0.14 us and a list of k = 50 that starts
+//                empty takes ~190 of them, so the CTAs first share a bound:
+//                each publishes its first tile's largest logit per query (or
+//                four, of 32 rows each), and the k-th largest over all CTAs,
+//                a bound on the k-th logit of the vocabulary, is waited for
+//                (at most kTcBoundWaitNs) before the first tile is entered;
+//                a few keys per query and CTA are left (128256 x 3072, k = 50:
+//                159.9 -> 140.1 us at 64 queries; e4m3 82.4 -> 74.5 us at 16,
+//                115.7 -> 83.3 us at 32).
 // Each CTA writes its per-query lists and takes a completion ticket; the
 // last CTAs to finish merge them, one query each.  All waits are bounded.
 //
@@ -61,6 +70,8 @@ constexpr int kTcListKeys = 4096;  // keys of the per-CTA lists per CTA: NQ * k 
 constexpr int kTcMaxKPS = 4;       // K-blocks per stage, at most
 constexpr int kTcMergeE = 8;       // merge: keys per list in the heads area
 constexpr int kQ8Pieces = 4;       // e4m3 columns per query on the Q8 path
+constexpr int kTcMaxSelWarps = 16;  // selector warps, at most
+constexpr uint64_t kTcBoundWaitNs = 20000;  // longest wait for the shared bound of the first tile
 constexpr int kTcMaxMergers = 64;  // CTAs that merge, at most (one per query)
 
 struct TcParams {
@@ -78,6 +89,9 @@ struct TcParams {
     uint32_t *next_tile;     // pool counter (self-resetting)
     uint32_t *epoch;         // launch counter word (advanced by the last CTA to finish)
     uint32_t *flags;         // [G] publication words: flags[c] = epoch + 1 once CTA c's lists are written
+    uint32_t *counts;        // [selector warps]: CTAs that have published their maxima (self-resetting)
+    int32_t gt_blocks;       // maxima each CTA publishes per query for the shared bound: 1, 4 or 0 (none)
+    uint64_t *gmax;          // [NQ][G][gt_blocks]: tag << 32 | the maximum's ordered logit
     uint32_t *err;           // device flag word
     int32_t *out_idx;        // [nq, k]
     float *out_logits;       // [nq, k]
@@ -179,8 +193,8 @@ __device__ __forceinline__ float e4m3_value(uint8_t c) {
 }
 
 // Keeps the k largest of the cnt (k < cnt <= 32 * PER) nonzero keys in buf, unsorted at
-// buf[0..k), and returns k; *tau becomes a bound T <= the k-th key such that
-// exactly k keys are >= T.  T is found by bisection: first on the high words
+// buf[0..k), and returns k; *tau becomes T - 1, T the k-th key (exactly k keys
+// are >= T).  T is found by bisection: first on the high words
 // (the logit order), then, only if several keys tie on the k-th high word,
 // on the low words (the row order) among the tied keys.  Out of line and
 // loop-based: a few hundred instructions, and little code next to the
@@ -246,7 +260,7 @@ static __device__ __noinline__ int keep_best(uint64_t *buf, int cnt, int k, uint
         if (in) buf[base + __popc(m & lt_mask)] = v[j];
         base += __popc(m);
     }
-    if (lane == 0) *tau = T;
+    if (lane == 0) *tau = T - 1;  // a key enters if it is above: T itself is kept, keys are unique
     __syncwarp();
     return k;
 }
@@ -254,8 +268,8 @@ static __device__ __noinline__ int keep_best(uint64_t *buf, int cnt, int k, uint
 // The final list of one query: the best min(k, cnt) keys of buf (cnt <=
 // 32 * CAP_PER), sorted descending, written to dst[0..k) (zeros after them),
 // and its first kTcMergeE keys also to head[0..kTcMergeE).  The sort network
-// spans 32 * PER keys, the least that holds k (k <= 32 * PER): its dependent
-// shuffles are the tail of the launch.
+// spans 32 * PER keys, the least that holds cnt or k (cnt <= 32 * PER or
+// k <= 32 * PER): its dependent shuffles are the tail of the launch.
 template <int CAP_PER, int PER>
 static __device__ __noinline__ void write_sorted_list(uint64_t *buf, int cnt, int k, uint64_t *tau,
                                                       uint64_t *dst, uint64_t *head, int lane) {
@@ -274,6 +288,7 @@ static __device__ __noinline__ void write_sorted_list(uint64_t *buf, int cnt, in
         if (e < k) dst[e] = v[j];
         if (e < kTcMergeE) head[e] = v[j];
     }
+    for (int e = 32 * PER + lane; e < k; e += 32) dst[e] = 0ull;
 }
 
 template <int NQ, bool Q8>
@@ -704,6 +719,24 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
             }
         }
         constexpr int QPW = Sh::kQPW;
+        static_assert(Sh::kSelWarps <= kTcMaxSelWarps, "a counter per selector warp");
+        // the shared bound: this CTA's maxima of query q over the first tile
+        const int gt = p.gt_blocks, n_max = G * gt;
+        const uint32_t tag = *reinterpret_cast<volatile uint32_t *>(p.epoch) + 1u;
+        auto publish_maxima = [&](int q, const float *scq, int64_t row0, int rows) {
+            uint32_t mx = 0;
+            for (int rb = 0; rb < rows; rb += 32) {
+                const int r = rb + lane;
+                const uint32_t hi = r < rows ? order_f32(scq[r]) : 0u;
+                mx = max(mx, __reduce_max_sync(0xFFFFFFFFu, hi));
+                if (gt == 4 || rb + 32 >= rows) {
+                    if (lane == 0)
+                        st_relaxed_gpu_u64(p.gmax + (static_cast<size_t>(q) * G + cta) * gt + (gt == 4 ? rb / 32 : 0),
+                                           (static_cast<uint64_t>(tag) << 32) | mx);
+                    mx = 0;
+                }
+            }
+        };
         if constexpr (Sh::kBufSel) {
             // per query of this warp: candidates above the bound tau in a shared
             // buffer, their count and tau next to it (only this warp touches them)
@@ -718,6 +751,22 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
             }
             __syncwarp();
             const unsigned lt_mask = (1u << lane) - 1u;
+            bool bounded = gt == 0;
+            // the bound, as far as the other CTAs have got: never waited for
+            auto look = [&]() {
+                bounded = true;
+#pragma unroll 1
+                for (int j = 0; j < QPW; ++j) {
+                    const int q = QPW * sel + j;
+                    if (q >= p.nq) break;
+                    const SharedBound sb =
+                        shared_bound(p.gmax + static_cast<size_t>(q) * n_max, n_max, tag, p.k, lane);
+                    if (lane == 0 && sb.bound != 0)
+                        tau_s[j] = max(tau_s[j], (static_cast<uint64_t>(sb.bound) << 32) - 1u);
+                    bounded = bounded && sb.n_valid == n_max;
+                }
+                __syncwarp();
+            };
             for (int ti = 0;; ++ti) {
                 const int ss = ti % SL, su = ti / SL;
                 if (!mbar_wait(&sfull[ss], su & 1, abort_flag)) {
@@ -732,10 +781,12 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                 const int64_t row0 = static_cast<int64_t>(rblk) * kTcTile;
                 const int rows = static_cast<int>(min(static_cast<int64_t>(kTcTile), p.V - row0));
                 const float *sc = scores + ss * NQ * kTcTile;
+                if (ti > 0 && !bounded) look();
 #pragma unroll 1
                 for (int j = 0; j < QPW; ++j) {
                     const int q = QPW * sel + j;
                     if (q >= p.nq) break;
+                    if (ti == 0 && gt > 0) publish_maxima(q, sc + q * kTcTile, row0, rows);
                     uint64_t *buf = buf0 + q * CAP;
                     int cnt = cnt_s[j];
                     uint64_t tau = tau_s[j];
@@ -760,6 +811,7 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
             }
             // this CTA's sorted top-k per query and its first keys -> scratch
             // (written even after a wait gave up: the merge then stays in bounds)
+            if (!bounded) look();
 #pragma unroll 1
             for (int j = 0; j < QPW; ++j) {
                 const int q = QPW * sel + j;
@@ -767,12 +819,13 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                 uint64_t *dst = p.cand + (static_cast<size_t>(q) * G + cta) * p.k;
                 uint64_t *head = p.heads + (static_cast<size_t>(q) * G + cta) * kTcMergeE;
                 uint64_t *buf = buf0 + q * CAP;
-                if (p.k <= 32)
-                    write_sorted_list<CAP_PER, 1>(buf, cnt_s[j], p.k, &tau_s[j], dst, head, lane);
-                else if (p.k <= 64)
-                    write_sorted_list<CAP_PER, 2>(buf, cnt_s[j], p.k, &tau_s[j], dst, head, lane);
+                const int cnt = warp_filter(buf, cnt_s[j], tau_s[j], lane);
+                if (cnt <= 32 || p.k <= 32)
+                    write_sorted_list<CAP_PER, 1>(buf, cnt, p.k, &tau_s[j], dst, head, lane);
+                else if (cnt <= 64 || p.k <= 64)
+                    write_sorted_list<CAP_PER, 2>(buf, cnt, p.k, &tau_s[j], dst, head, lane);
                 else
-                    write_sorted_list<CAP_PER, kTcMaxK / 32>(buf, cnt_s[j], p.k, &tau_s[j], dst, head, lane);
+                    write_sorted_list<CAP_PER, kTcMaxK / 32>(buf, cnt, p.k, &tau_s[j], dst, head, lane);
             }
         } else {
             // per query of this warp: its best keys so far as a sorted list spread
@@ -795,6 +848,42 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                     break;
                 }
                 const int rblk = mc->slot_tile[ss];
+                if (ti == 0 && gt > 0) {
+                    // every CTA counts itself, with or without a tile
+                    const float *sc0 = scores + ss * NQ * kTcTile;
+                    const int64_t r0 = static_cast<int64_t>(rblk) * kTcTile;
+                    if (rblk >= 0) {
+#pragma unroll 1
+                        for (int j = 0; j < QPW; ++j) {
+                            const int q = QPW * sel + j;
+                            if (q < p.nq)
+                                publish_maxima(q, sc0 + q * kTcTile, r0,
+                                               static_cast<int>(min(static_cast<int64_t>(kTcTile), p.V - r0)));
+                        }
+                    }
+                    if (lane == 0) {
+                        red_add_release_gpu(p.counts + sel, 1u);
+                        __threadfence();  // performed before this CTA's ticket, after which it may be re-armed
+                    }
+                    if (rblk >= 0) {
+                        if (lane == 0) {
+                            const uint64_t t0 = global_timer_ns();
+                            while (ld_acquire_gpu(p.counts + sel) < static_cast<uint32_t>(G) &&
+                                   global_timer_ns() - t0 < kTcBoundWaitNs && !*abort_flag) {
+                            }
+                        }
+                        __syncwarp();
+#pragma unroll
+                        for (int j = 0; j < QPW; ++j) {
+                            const int q = QPW * sel + j;
+                            if (q < p.nq) {
+                                const SharedBound sb =
+                                    shared_bound(p.gmax + static_cast<size_t>(q) * n_max, n_max, tag, p.k, lane);
+                                if (sb.bound != 0) tau[j] = (static_cast<uint64_t>(sb.bound) << 32) - 1u;
+                            }
+                        }
+                    }
+                }
                 if (rblk < 0) break;
                 const int64_t row0 = static_cast<int64_t>(rblk) * kTcTile;
                 const int rows = static_cast<int>(min(static_cast<int64_t>(kTcTile), p.V - row0));
@@ -818,7 +907,7 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                                     m &= m - 1;
                                     list[j].insert(shfl_u64(key, src), lane);
                                 } while (m);
-                                tau[j] = list[j].at(p.k - 1);
+                                tau[j] = max(tau[j], list[j].at(p.k - 1));
                             }
                         }
                     }
@@ -864,9 +953,10 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
     if (tid == 0) {
         st_release_gpu(p.flags + cta, target);
         const uint32_t ticket = atomic_add_relaxed_gpu(p.ticket, 1u);
-        if (ticket == static_cast<uint32_t>(G - 1)) {
+        if (ticket == static_cast<uint32_t>(G - 1)) {  // (every selector has counted itself by then)
             *p.next_tile = 0;
             *p.ticket = 0;
+            for (int i = 0; i < Sh::kSelWarps; ++i) p.counts[i] = 0;
             *reinterpret_cast<volatile uint32_t *>(p.epoch) = target;
         }
         mc->merger = ticket < static_cast<uint32_t>(X) ? static_cast<int>(ticket) : -1;
