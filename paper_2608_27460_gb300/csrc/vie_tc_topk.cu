@@ -12,6 +12,7 @@ namespace vie {
 __global__ void prep_queries_kernel(const float *__restrict__ h, int nq, int d, int d_pad,
                                     int n_rows, __nv_bfloat16 *__restrict__ hB) {
     griddep_launch_dependents();  // the projection kernel may start its prologue now
+    griddep_wait();  // h comes from the kernel before this one, which may still read hB
     const int64_t n = static_cast<int64_t>(n_rows) * d_pad;
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -122,9 +123,8 @@ cudaError_t launch_prep_queries(const float *h, int nq, int d, int d_pad, int n_
     const int64_t n = static_cast<int64_t>(n_rows) * d_pad;
     int64_t blocks = (n + 255) / 256;
     if (blocks > 4LL * sms) blocks = 4LL * sms;
-    prep_queries_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
-        h, nq, d, d_pad, n_rows, static_cast<__nv_bfloat16 *>(hB));
-    return cudaGetLastError();
+    return launch_pdl(prep_queries_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, stream, h, nq, d,
+                      d_pad, n_rows, static_cast<__nv_bfloat16 *>(hB));
 }
 
 }  // namespace vie
