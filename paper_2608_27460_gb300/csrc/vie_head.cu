@@ -17,6 +17,7 @@
 
 #include "vie_head.h"
 #include "vie_launch.h"
+#include "vie_tc_many.cuh"
 #include "vie_tc_topk.cuh"
 
 namespace {
@@ -59,6 +60,9 @@ constexpr int kNumWords = kCountWords + vie::kTcMaxSelWarps;
 // Words per CTA of the shared bounds' maxima (gmax): 8 queries x 8 on the
 // streaming path, 64 x 1 or 32 x 4 on the tensor-core path.
 constexpr int kBoundWords = 128;
+// Rows of a bf16 head's query matrix: hi and lo of a block of many queries.
+constexpr int kHRows = 2 * vie::kMnBlock;
+static_assert(kHRows >= vie::kTcHRows, "the batched path's query matrix fits");
 
 }  // namespace
 
@@ -72,14 +76,20 @@ struct vie_head {
     float *scale;       // e4m3 heads: fp32 scale per row [V]; nullptr for bf16 heads
     uint64_t *cand;     // [kMaxNB][G][VIE_K_MAX] ranking keys, then [kMaxNB][G][kWideE] heads
     uint32_t *words;    // kNumWords scratch words (see kEpochWord, kFlagWords)
-    uint64_t *gmax;     // [G * kBoundWords] maxima behind the shared bounds (tagged words)
+    uint64_t *gmax;     // [G * kBoundWords] maxima behind the shared bounds (tagged words), in cand's allocation
     int64_t scratch_bytes;
     // tensor-core path (batches): hi/lo bf16 query matrix and TMA descriptors
-    void *hB;             // [kTcHRows][d_pad] bf16, or e4m3 query pieces [4 NQ][d_pad]
+    void *hB;             // [kHRows][d_pad] bf16, or e4m3 query pieces [4 NQ][d_pad]
     float *qscale;        // e4m3 heads: [32][kQ8Pieces] piece scales of the query group
     bool tc_ready;
     CUtensorMap mapW;     // W as [V][d_pad], box 128 rows x 128 bytes, 128-byte swizzle
     CUtensorMap mapH[4];  // hB, box 16 / 32 / 64 / 128 rows x 128 bytes
+    // many queries (bf16 heads): the sample's logits and then the candidates
+    // of a block of queries lie in cand, their bounds and counts behind gmax
+    bool many_ready;
+    size_t cand_bytes;
+    CUtensorMap mapHM;     // hB, all kHRows rows, box 128 rows x 128 bytes
+    CUtensorMap mapS[4];   // every 8th / 16th / 32nd / 64th row of W, box as mapW
     // vie_head_topk_host: device staging of queries and top-k (grown on demand)
     float *stage_h;
     int32_t *stage_idx;
@@ -344,6 +354,43 @@ bool make_map_bf16(CUtensorMap *m, void *base, uint64_t rows, uint64_t cols, uin
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Batches of at least this many queries run as a filtered GEMM.  Below it the
+// batched path's passes over W (64 queries each) cost less than a block's five
+// launches and its sample.
+constexpr int kManyMinBatch = 256;
+constexpr int64_t kManyMinRows = 8192;  // a smaller vocabulary's sample bounds too little
+
+// The sample takes every (8 << i)-th row: the widest stride, 64 at most, with
+// which the candidates of a query (k times the stride on average, within a
+// factor 1 +- 1 / sqrt(k)) stay below kMnCap for all but one query in 10^6.
+int many_stride_log2(int k) { return k <= 8 ? 3 : (k <= 20 ? 2 : (k <= 64 ? 1 : 0)); }
+
+int64_t many_pitch(const vie_head *hd, int k) {
+    const int64_t st = 8 << many_stride_log2(k);
+    return ((hd->V + st - 1) / st + 31) / 32 * 32;
+}
+
+// Queries of a block of launches: whole groups whose sample fits the scratch
+// (0: not even one).
+int many_block(const vie_head *hd, int k) {
+    const int64_t n = static_cast<int64_t>(hd->cand_bytes) / (many_pitch(hd, k) * 4) / vie::kMnGroup * vie::kMnGroup;
+    return static_cast<int>(n < vie::kMnBlock ? n : vie::kMnBlock);
+}
+
+// Sets up a bf16 head for many queries, in scratch that the other paths use
+// between such calls.
+void init_many(vie_head *hd) {
+    hd->many_ready = hd->tc_ready && hd->V >= kManyMinRows && hd->d_pad >= 64 && hd->num_sms >= 2 &&
+                     hd->cand_bytes >= vie::kMnBlock * vie::kMnCap * sizeof(uint64_t);
+    const uint64_t pitch = static_cast<uint64_t>(hd->d_pad) * 2;
+    if (hd->many_ready) hd->many_ready = make_map_bf16(&hd->mapHM, hd->hB, kHRows, hd->d_pad, pitch, 128);
+    for (int i = 0; i < 4 && hd->many_ready; ++i) {
+        const uint64_t st = 8u << i;
+        hd->many_ready =
+            make_map_bf16(&hd->mapS[i], hd->W, (static_cast<uint64_t>(hd->V) + st - 1) / st, hd->d_pad, pitch * st, 128);
+    }
+}
+
 }  // namespace
 
 extern "C" {
@@ -419,16 +466,18 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
     const size_t cbytes =
         static_cast<size_t>(kMaxNB) * hd->G * (VIE_K_MAX + vie::kWideE) * sizeof(uint64_t);
     const size_t gbytes = static_cast<size_t>(hd->G) * kBoundWords * sizeof(uint64_t);
-    hd->scratch_bytes = static_cast<int64_t>(cbytes + gbytes + kNumWords * sizeof(uint32_t));
+    const size_t mbytes = static_cast<size_t>(vie::kMnBlock) * (sizeof(uint64_t) + 2 * sizeof(float));
+    hd->cand_bytes = cbytes;
+    hd->scratch_bytes = static_cast<int64_t>(cbytes + gbytes + mbytes + kNumWords * sizeof(uint32_t));
     e = cudaMalloc(&hd->W, wbytes);
     if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->scale, static_cast<size_t>(V) * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&hd->cand, cbytes);
-    if (e == cudaSuccess) e = cudaMemset(hd->cand, 0, cbytes);  // empty lists until written
-    if (e == cudaSuccess) e = cudaMalloc(&hd->gmax, gbytes);
-    if (e == cudaSuccess) e = cudaMemset(hd->gmax, 0, gbytes);  // tag 0: of no launch
+    if (e == cudaSuccess) e = cudaMalloc(&hd->cand, cbytes + gbytes + mbytes);
+    // bounds of no launch (tag 0); empty lists until written
+    if (e == cudaSuccess) e = cudaMemset(hd->cand, 0, cbytes + gbytes + mbytes);
+    if (e == cudaSuccess) hd->gmax = hd->cand + cbytes / sizeof(uint64_t);
     if (e == cudaSuccess) e = cudaMalloc(&hd->words, kNumWords * sizeof(uint32_t));
     if (e == cudaSuccess)
-        e = cudaMalloc(&hd->hB, static_cast<size_t>(vie::kTcHRows) * hd->d_pad * 2);
+        e = cudaMalloc(&hd->hB, static_cast<size_t>(e4m3 ? vie::kTcHRows : kHRows) * hd->d_pad * 2);
     if (e == cudaSuccess) e = cudaMemset(hd->hB, 0, static_cast<size_t>(vie::kTcHRows) * hd->d_pad * 2);
     if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->qscale, 32 * vie::kQ8Pieces * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(hd->words, 0, kNumWords * sizeof(uint32_t));
@@ -453,7 +502,6 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
         cudaFree(hd->W);
         cudaFree(hd->scale);
         cudaFree(hd->cand);
-        cudaFree(hd->gmax);
         cudaFree(hd->words);
         cudaFree(hd->hB);
         cudaFree(hd->qscale);
@@ -474,6 +522,7 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
                                  vie::kTcTile);
     for (int i = 0; i < 4 && hd->tc_ready; ++i)
         hd->tc_ready = make_map_bf16(&hd->mapH[i], hd->hB, vie::kTcHRows, hd->d_pad, pitch, 16u << i);
+    init_many(hd);
     *out = hd;
     return VIE_OK;
 }
@@ -511,7 +560,6 @@ vie_status vie_head_destroy(vie_head *head) {
     cudaFree(head->W);
     cudaFree(head->scale);
     cudaFree(head->cand);
-    cudaFree(head->gmax);
     cudaFree(head->words);
     cudaFree(head->hB);
     cudaFree(head->qscale);
@@ -554,6 +602,11 @@ static bool use_tc(const vie_head *head, int32_t batch, int32_t k) {
            k <= vie::tc_max_k(32, q8) && head->d_pad >= (q8 ? 128 : 64);
 }
 
+static bool use_many(const vie_head *head, int32_t batch, int32_t k) {
+    return head->many_ready && batch >= kManyMinBatch && k <= vie::kMnMaxK && use_tc(head, batch, k) &&
+           many_block(head, k) > 0;
+}
+
 // Bytes of the query operand each CTA of a group of nqt slots builds itself
 // (0: a prep kernel writes it).
 static int tc_hres(const vie_head *head, int nqt) {
@@ -564,7 +617,12 @@ static int tc_hres(const vie_head *head, int nqt) {
 
 static vie_topk_plan make_plan(const vie_head *head, int32_t batch, int32_t k) {
     vie_topk_plan pl;
-    if (use_tc(head, batch, k)) {
+    if (use_many(head, batch, k)) {
+        const int block = many_block(head, k);
+        pl.path = 1;
+        pl.groups = (batch + vie::kMnGroup - 1) / vie::kMnGroup;
+        pl.launches = 5 * ((batch + block - 1) / block);  // prep, sample, bounds, main, final
+    } else if (use_tc(head, batch, k)) {
         const int nqt = tc_group(batch, k, head->scale != nullptr);
         pl.path = 1;
         pl.groups = (batch + nqt - 1) / nqt;
@@ -647,6 +705,48 @@ static vie_status run_topk_tc(const char *fn, vie_head *head, const float *h, in
     return VIE_OK;
 }
 
+// Many queries: blocks of the filtered GEMM (vie_tc_many.cuh).
+static vie_status run_topk_many(const char *fn, vie_head *head, const float *h, int32_t batch, int32_t k,
+                                int32_t *out_idx, float *out_logits, float *sparse, cudaStream_t s) {
+    const int si = many_stride_log2(k), stride = 8 << si, block = many_block(head, k);
+    const int rows = static_cast<int>((head->V + stride - 1) / stride);
+    const int64_t pitch = many_pitch(head, k);
+    float *sample = reinterpret_cast<float *>(head->cand);  // read for the bounds before candidates replace it
+    uint64_t *tau = head->gmax + static_cast<size_t>(head->G) * kBoundWords;
+    float *tau_v = reinterpret_cast<float *>(tau + vie::kMnBlock);
+    uint32_t *count = reinterpret_cast<uint32_t *>(tau_v + vie::kMnBlock);
+    for (int q0 = 0; q0 < batch; q0 += block) {
+        const int nq = batch - q0 < block ? batch - q0 : block;
+        const int groups = (nq + vie::kMnGroup - 1) / vie::kMnGroup;
+        const float *hq = h + static_cast<int64_t>(q0) * head->d;
+        vie::MnParams p;
+        p.d_pad = head->d_pad;
+        p.groups = groups;
+        p.tau = tau;
+        p.tau_v = tau_v;
+        p.cand = head->cand;
+        p.count = count;
+        p.err = head->words + 1;
+        cudaError_t e = vie::launch_prep_queries(hq, nq, head->d, head->d_pad, groups * 2 * vie::kMnGroup, head->hB,
+                                                 head->num_sms, s);
+        p.rows = rows;
+        p.sample = sample;
+        p.sample_pitch = pitch;
+        if (e == cudaSuccess) e = vie::launch_tc_many(head->mapS[si], head->mapHM, p, head->num_sms, s);
+        if (e == cudaSuccess)
+            e = vie::launch_many_tau(sample, pitch, rows, stride, nq, groups * vie::kMnGroup, k, tau, tau_v, count, s);
+        p.rows = head->V;
+        p.sample = nullptr;
+        if (e == cudaSuccess) e = vie::launch_tc_many(head->mapW, head->mapHM, p, head->num_sms, s);
+        if (e == cudaSuccess)
+            e = vie::launch_many_final(head->cand, count, nq, k, head->W, head->V, head->d, head->d_pad, hq,
+                                       out_idx + static_cast<int64_t>(q0) * k, out_logits + static_cast<int64_t>(q0) * k,
+                                       sparse != nullptr ? sparse + static_cast<int64_t>(q0) * head->V : nullptr, s);
+        if (e != cudaSuccess) return fail_cuda(e, fn);
+    }
+    return VIE_OK;
+}
+
 static vie_status run_topk(const char *fn, vie_head *head, const float *h, int32_t batch,
                            int32_t k, int32_t *out_idx, float *out_logits, float *sparse,
                            vie_stream stream) {
@@ -665,6 +765,7 @@ static vie_status run_topk(const char *fn, vie_head *head, const float *h, int32
     if (st != VIE_OK) return st;
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (use_many(head, batch, k)) return run_topk_many(fn, head, h, batch, k, out_idx, out_logits, sparse, s);
     if (use_tc(head, batch, k)) return run_topk_tc(fn, head, h, batch, k, out_idx, out_logits, sparse, s);
     const int row_bytes = head->d_pad * (head->scale != nullptr ? 1 : 2);
     // published wide lists: the merge stages kWideE keys of every list

@@ -1096,7 +1096,7 @@ __device__ inline void merge_queries(const uint64_t *cand, const uint64_t *heads
 // kFastE of the top k, or fewer than k real heads) the lists (lists_q, G x k
 // keys) are merged in full.  ws holds the merge buffers (merge_fixed_bytes);
 // fe holds G * kFastE keys and then ceil(G/8)*8 head words.  Every wait is
-// bounded; a list that never arrives is reported in *err and counted empty.
+// bounded; a list that never arrives is reported in *err and nothing is written.
 __device__ inline void merge_published(const uint32_t *flags, uint32_t target, const uint64_t *heads_q,
                                        const uint64_t *lists_q, int G, int k, unsigned char *ws,
                                        uint64_t *fe, MiscSmem *ms, uint32_t *err, int32_t *oi, float *ol,
@@ -1119,6 +1119,7 @@ __device__ inline void merge_published(const uint32_t *flags, uint32_t target, c
     merge_fast_reset(mb.counts, ms);
     bool pending = tid < G;  // thread c watches list c
     bool have = false;       // list c seen, its heads not copied yet
+    bool missing = false;    // list c never came
     const uint64_t t0 = global_timer_ns();
     for (;;) {
         const bool load_now = have;
@@ -1134,6 +1135,7 @@ __device__ inline void merge_published(const uint32_t *flags, uint32_t target, c
                 have = true;
             } else if (global_timer_ns() - t0 > kWaitLimitNs) {
                 pending = false;
+                missing = true;
                 atomicOr(err, kErrWaitTimeout);
             }
         }
@@ -1145,6 +1147,7 @@ __device__ inline void merge_published(const uint32_t *flags, uint32_t target, c
         }
         if (__syncthreads_count((pending || have) ? 1 : 0) == 0) break;
     }
+    if (__syncthreads_or(missing ? 1 : 0)) return;  // no list to merge there: no output, the flag tells
     // every list is in: the barrier above ordered each thread's acquire (and
     // the fast merge's reset) before what follows
     const bool fast_ok = k <= G && 2 * G <= static_cast<int>(blockDim.x);
@@ -1184,6 +1187,7 @@ __device__ inline void merge_published_wide(const uint32_t *flags, uint32_t targ
         ms->overflow = 0;
         ms->remaining = 0;
     }
+    bool missing = false;
     const uint64_t t0 = global_timer_ns();
     for (bool pending = tid < G;;) {
         if (pending) {
@@ -1191,11 +1195,13 @@ __device__ inline void merge_published_wide(const uint32_t *flags, uint32_t targ
                 pending = false;
             } else if (global_timer_ns() - t0 > kWaitLimitNs) {
                 pending = false;
+                missing = true;
                 atomicOr(err, kErrWaitTimeout);
             }
         }
         if (__syncthreads_count(pending ? 1 : 0) == 0) break;
     }
+    if (__syncthreads_or(missing ? 1 : 0)) return;
     // 1. the heads, staged with one key of padding per list (thread c then
     // walks list c without bank conflicts)
     const int n_heads = G * kWideE;

@@ -1,0 +1,367 @@
+// vie_tc_many.cu - the filtered GEMM for many queries (vie_tc_many.cuh), the
+// bounds from its sample, the final top-k of each query's candidates, and
+// their launchers.
+#include "vie_launch.h"
+#include "vie_stream_topk.cuh"
+#include "vie_tc_launch.cuh"
+#include "vie_tc_many.cuh"
+#include "vie_tcgen05.cuh"
+
+namespace vie {
+
+struct MnMisc {
+    uint32_t tmem_base;
+    int abort;
+};
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMnThreads, 1)
+    tc_many_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapH,
+                   const MnParams p) {
+    extern __shared__ __align__(1024) unsigned char mn_smem[];
+    uint64_t *full = reinterpret_cast<uint64_t *>(mn_smem);
+    uint64_t *empty = full + kMnStages;
+    uint64_t *tfull = empty + kMnStages;
+    uint64_t *tempty = tfull + 2;
+    uint64_t *final_bar = tempty + 2;
+    MnMisc *mc = reinterpret_cast<MnMisc *>(mn_smem + 512);
+    unsigned char *ring = mn_smem + 1024;
+    ring += (1024u - (smem_addr(ring) & 1023u)) & 1023u;
+    volatile int *abort_flag = &mc->abort;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t rank = cluster_ctarank();
+    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    const int n_kb = (p.d_pad + 63) / 64;
+    const int n_items = static_cast<int>((p.rows + kMnRows - 1) / kMnRows) * p.groups;
+
+    if (tid == 0) {
+        for (int s = 0; s < kMnStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&tfull[b], 1);
+            mbar_init(&tempty[b], 2 * kMnEpiWarps);
+        }
+        mbar_init(final_bar, 1);
+        mc->abort = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc_pair(&mc->tmem_base, 512);
+        tmem_relinquish_pair();
+        tc_fence_before_sync();
+    }
+    __syncthreads();
+    cluster_sync();  // the pair's barriers are set up before either CTA signals the other's
+    tc_fence_after_sync();
+    const uint32_t tmem = mc->tmem_base;
+    if (tid == 0) griddep_launch_dependents();
+
+    // Items in order: the groups of one tile of W are neighbours, so that the
+    // pairs that run them together read the tile from HBM once.
+    if (warp == 0) {
+        // ---------------- TMA producer ----------------
+        if (lane == 0) {
+            tma_prefetch_map(&mapW);
+            tma_prefetch_map(&mapH);
+            griddep_wait();  // the query matrix comes from the kernel before this one
+            int it = 0, issued = 0;
+            bool ok = true;
+            for (int item = pair; item < n_items && ok; item += n_pairs) {
+                const int tile = item / p.groups, g = item - tile * p.groups;
+                for (int kb = 0; kb < n_kb; ++kb, ++it) {
+                    const int s = it % kMnStages, u = it / kMnStages;
+                    if (it >= kMnStages && !mbar_wait(&empty[s], (u - 1) & 1, abort_flag)) {
+                        ok = false;
+                        break;
+                    }
+                    unsigned char *st = ring + s * kMnStageBytes;
+                    if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * kMnStageBytes);
+                    const uint32_t bar = cluster_map(&full[s], 0);
+                    tma_load_2d_pair(st, &mapW, kb * 64, tile * kMnRows + static_cast<int>(rank) * 128, bar);
+                    tma_load_2d_pair(st + kMnStageBytes / 2, &mapH, kb * 64,
+                                     g * 2 * kMnGroup + static_cast<int>(rank) * 128, bar);
+                    issued = it + 1;
+                }
+            }
+            if (!ok) {
+                atomicOr(p.err, kErrWaitTimeout);
+                mc->abort = 1;
+                // copies in flight land before the CTA exits: the leader can
+                // watch its barriers, the other CTA gives them a millisecond
+                const int never = 0;
+                if (rank == 0)
+                    for (int t2 = max(0, issued - kMnStages); t2 < issued; ++t2)
+                        mbar_wait(&full[t2 % kMnStages], (t2 / kMnStages) & 1, const_cast<volatile int *>(&never));
+                const uint64_t t0 = global_timer_ns();
+                while (global_timer_ns() - t0 < 1000000ull) {
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (the leader's) ----------------
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = umma_idesc_bf16_f32(kMnRows, 2 * kMnGroup);
+            int it = 0, ti = 0;
+            bool ok = true;
+            for (int item = pair; item < n_items && ok; item += n_pairs, ++ti) {
+                const int b = ti & 1, ub = ti >> 1;
+                if (ti >= 2 && !mbar_wait(&tempty[b], (ub - 1) & 1, abort_flag)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after_sync();
+                const uint32_t d = tmem + static_cast<uint32_t>(b * 2 * kMnGroup);
+                for (int kb = 0; kb < n_kb; ++kb, ++it) {
+                    const int s = it % kMnStages, u = it / kMnStages;
+                    if (!mbar_wait(&full[s], u & 1, abort_flag)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after_sync();
+                    unsigned char *st = ring + s * kMnStageBytes;
+                    const uint64_t ad = umma_desc_k_sw128(st), bd = umma_desc_k_sw128(st + kMnStageBytes / 2);
+#pragma unroll
+                    for (int k4 = 0; k4 < 4; ++k4)
+                        umma_bf16_pair(d, ad + 2 * k4, bd + 2 * k4, idesc, (kb | k4) != 0 ? 1u : 0u);
+                    umma_commit_pair(&empty[s]);
+                }
+                if (ok) umma_commit_pair(&tfull[b]);
+            }
+            if (!ok) {
+                atomicOr(p.err, kErrWaitTimeout);
+                mc->abort = 1;
+            }
+            // every MMA this thread issued has finished before TMEM is freed
+            umma_commit_pair_local(final_bar);
+            const int never = 0;
+            mbar_wait(final_bar, 0, const_cast<volatile int *>(&never));
+        }
+        __syncwarp();
+    } else {
+        // ---------------- epilogue ----------------
+        griddep_wait();  // the bounds; and the outputs follow the previous kernel
+        const int qw = warp & 3, half = (warp - 2) >> 2;
+        const unsigned row_in_tile = rank * 128u + 32u * qw + lane;
+        int ti = 0;
+        for (int item = pair; item < n_items; item += n_pairs, ++ti) {
+            const int tile = item / p.groups, g = item - tile * p.groups;
+            const int b = ti & 1, ub = ti >> 1;
+            if (!mbar_wait(&tfull[b], ub & 1, abort_flag)) {
+                if (lane == 0) {
+                    atomicOr(p.err, kErrWaitTimeout);
+                    mc->abort = 1;
+                }
+                break;
+            }
+            tc_fence_after_sync();
+            const int64_t row = static_cast<int64_t>(tile) * kMnRows + row_in_tile;
+            const bool real = row < p.rows;
+            const uint32_t tb = tmem + (static_cast<uint32_t>(32 * qw) << 16) + b * 2 * kMnGroup + half * kMnGroup;
+            const int q0 = g * kMnGroup + half * (kMnGroup / 2);
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {  // 32 columns, 16 queries
+                uint32_t r[2][16];
+                tmem_ld_32x32b_x16(tb + 32 * c, r[0]);
+                tmem_ld_32x32b_x16(tb + 32 * c + 16, r[1]);
+                tmem_wait_ld();
+                float z[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    z[i] = __uint_as_float(r[i / 8][2 * (i % 8)]) + __uint_as_float(r[i / 8][2 * (i % 8) + 1]);
+                const int q = q0 + 16 * c;
+                if (p.sample != nullptr) {
+                    if (real) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) p.sample[(q + i) * p.sample_pitch + row] = z[i];
+                    }
+                    continue;
+                }
+                uint32_t in = 0;
+                const float4 *t4 = reinterpret_cast<const float4 *>(p.tau_v + q);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 t = t4[i];
+                    in |= (z[4 * i] >= t.x ? 1u : 0u) << (4 * i);
+                    in |= (z[4 * i + 1] >= t.y ? 1u : 0u) << (4 * i + 1);
+                    in |= (z[4 * i + 2] >= t.z ? 1u : 0u) << (4 * i + 2);
+                    in |= (z[4 * i + 3] >= t.w ? 1u : 0u) << (4 * i + 3);
+                }
+                if (!real) in = 0;
+                if (__any_sync(0xFFFFFFFFu, in != 0)) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        if (in >> i & 1u) {
+                            const uint64_t key = make_key(z[i], static_cast<uint32_t>(row));
+                            if (key >= p.tau[q + i]) {
+                                const uint32_t pos = atomicAdd(p.count + q + i, 1u);
+                                if (pos < kMnCap) p.cand[static_cast<size_t>(q + i) * kMnCap + pos] = key;
+                            }
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(cluster_map(&tempty[b], 0));
+        }
+    }
+
+    __syncthreads();
+    cluster_sync();  // neither CTA signals the other any more, and its operands are no longer read
+    if (warp == 1) {
+        tc_fence_after_sync();
+        tmem_dealloc_pair(tmem, 512);
+    }
+}
+
+namespace {
+
+// Keys of the sampled rows of one query: logit z[i] of vocabulary row i * stride.
+struct SampleKeys {
+    const float *z;
+    uint32_t stride;
+    __device__ __forceinline__ uint64_t operator[](int i) const {
+        return make_key(z[i], static_cast<uint32_t>(i) * stride);
+    }
+};
+
+}  // namespace
+
+// One CTA per query slot of the block: tau[q] = a key with exactly k sampled
+// keys at or above it, tau_v[q] its logit (+inf for slots without a query, so
+// that none of their logits pass), count[q] = 0.
+__global__ void __launch_bounds__(256) many_tau_kernel(const float *__restrict__ sample, int64_t pitch, int rows,
+                                                       uint32_t stride, int nq, int k, uint64_t *tau, float *tau_v,
+                                                       uint32_t *count) {
+    __shared__ uint32_t hist[256];
+    __shared__ MiscSmem ms;
+    griddep_launch_dependents();
+    griddep_wait();
+    const int q = blockIdx.x;
+    uint64_t t = ~0ull;
+    if (q < nq) t = block_radix_threshold(SampleKeys{sample + q * pitch, stride}, rows, k, 1, hist, &ms);
+    if (threadIdx.x == 0) {
+        const uint32_t hi = static_cast<uint32_t>(t >> 32);
+        tau[q] = t;
+        // (below order_f32(-FLT_MAX) there are only -inf and NaN patterns)
+        tau_v[q] = q >= nq ? __uint_as_float(0x7F800000u) : (hi < 0x00800000u ? __uint_as_float(0xFF800000u) : unorder_f32(hi));
+        count[q] = 0;
+    }
+}
+
+// One CTA per query: the exact top-k of its candidates, best first, and its
+// row of the sparse tensor.  A list that overflowed is replaced by the best of
+// all rows, computed here (fp32 dot products, one warp per row).
+__global__ void __launch_bounds__(kThreads) many_final_kernel(const uint64_t *cand, const uint32_t *count,
+                                                             int k, const uint16_t *W,
+                                                             int64_t V, int d, int d_pad, const float *h,
+                                                             int32_t *out_idx, float *out_logits, float *sparse) {
+    extern __shared__ __align__(16) unsigned char fin_smem[];
+    __shared__ MiscSmem ms;
+    MergeBufs mb;
+    mb.pref = reinterpret_cast<uint64_t *>(fin_smem);
+    mb.cands = mb.pref + kMergePrefixCap;
+    mb.win = mb.cands + kMergeCandCap;
+    mb.counts = reinterpret_cast<int *>(mb.win + 1024);
+    mb.offsets = mb.counts + kMaxLists;
+    mb.hist = reinterpret_cast<uint32_t *>(mb.offsets + kMaxLists);
+    griddep_launch_dependents();
+    griddep_wait();
+    const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float *sp = nullptr;
+    if (sparse != nullptr) {
+        sp = sparse + q * V;
+        for (int64_t i = tid; i < V; i += kThreads) sp[i] = __uint_as_float(0xFF800000u);
+    }
+    const uint64_t *list = cand + static_cast<size_t>(q) * kMnCap;
+    const uint32_t n_all = count[q];
+    if (tid == 0) {
+        ms.n_win = 0;
+        ms.n_cand = 0;
+    }
+    __syncthreads();
+    static_assert(kMnCap <= kMergeCandCap, "a query's candidates are ranked in shared memory");
+    int n;
+    if (n_all >= static_cast<uint32_t>(k) && n_all <= kMnCap) {
+        n = static_cast<int>(n_all);
+        for (int i = tid; i < n; i += kThreads) mb.cands[i] = __ldcg(reinterpret_cast<const unsigned long long *>(list) + i);
+    } else {
+        const float *hq = h + static_cast<int64_t>(q) * d;
+        constexpr int kRound = kMergeCandCap / 2;  // rows between cut-backs; k <= 1024 stay
+        uint64_t bound = 1;  // (tau is a tensor-core logit: these sums may fall a rounding short of it)
+        for (int64_t r0 = 0; r0 < V; r0 += kRound) {
+            const int64_t r1 = min(V, r0 + kRound);
+            for (int64_t r = r0 + warp; r < r1; r += kThreads / 32) {
+                const uint16_t *wr = W + r * d_pad;
+                float a = 0.0f;
+                for (int j = lane; j < d; j += 32) a = fmaf(__uint_as_float(static_cast<uint32_t>(wr[j]) << 16), hq[j], a);
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
+                const uint64_t key = make_key(a, static_cast<uint32_t>(r));
+                if (lane == 0 && key >= bound) mb.cands[atomicAdd(&ms.n_cand, 1)] = key;
+            }
+            __syncthreads();
+            const int m = ms.n_cand;
+            __syncthreads();  // read by all before the next round adds to it
+            if (m > kMergeCandCap / 2) {  // keep the best k
+                const uint64_t T = block_radix_threshold(SmemKeys{mb.cands}, m, k, 1, mb.hist, &ms);
+                for (int i = tid; i < m; i += kThreads)
+                    if (mb.cands[i] >= T) mb.win[atomicAdd(&ms.n_win, 1)] = mb.cands[i];
+                __syncthreads();
+                for (int i = tid; i < k; i += kThreads) mb.cands[i] = mb.win[i];
+                bound = T;
+                __syncthreads();
+                if (tid == 0) {
+                    ms.n_win = 0;
+                    ms.n_cand = k;
+                }
+                __syncthreads();
+            }
+        }
+        n = ms.n_cand;
+    }
+    __syncthreads();
+    block_topk_to_output(mb.cands, n, k, mb, &ms, out_idx + static_cast<int64_t>(q) * k,
+                         out_logits + static_cast<int64_t>(q) * k, sp);
+}
+
+cudaError_t launch_tc_many(const CUtensorMap &mapW, const CUtensorMap &mapH, const MnParams &p, int sms,
+                           cudaStream_t stream) {
+    static bool configured[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!configured[dev]) {
+        e = cudaFuncSetAttribute(tc_many_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMnSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(many_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     SmemLayout::merge_fixed_bytes());
+        if (e != cudaSuccess) return e;
+        configured[dev] = true;
+    }
+    int64_t pairs = (p.rows + kMnRows - 1) / kMnRows * p.groups;
+    if (pairs > sms / 2) pairs = sms / 2;
+    return launch_pdl(tc_many_kernel, dim3(static_cast<unsigned>(2 * pairs)), dim3(kMnThreads), kMnSmem, stream, mapW,
+                      mapH, p);
+}
+
+cudaError_t launch_many_tau(const float *sample, int64_t pitch, int rows, int stride, int nq, int slots, int k,
+                            uint64_t *tau, float *tau_v, uint32_t *count, cudaStream_t stream) {
+    return launch_pdl(many_tau_kernel, dim3(static_cast<unsigned>(slots)), dim3(256), 0, stream, sample, pitch, rows,
+                      static_cast<uint32_t>(stride), nq, k, tau, tau_v, count);
+}
+
+cudaError_t launch_many_final(const uint64_t *cand, const uint32_t *count, int nq, int k,
+                              const void *W, int64_t V, int d, int d_pad, const float *h, int32_t *out_idx,
+                              float *out_logits, float *sparse, cudaStream_t stream) {
+    return launch_pdl(many_final_kernel, dim3(static_cast<unsigned>(nq)), dim3(kThreads),
+                      SmemLayout::merge_fixed_bytes(), stream, cand, count, k,
+                      static_cast<const uint16_t *>(W), V, d, d_pad, h, out_idx, out_logits, sparse);
+}
+
+}  // namespace vie

@@ -77,3 +77,31 @@ def test_all_rows_equal_full_groups(vie):
         idx, val = run_head(vie, W, h, k)
         np.testing.assert_array_equal(idx, np.tile(np.arange(k, dtype=np.int32), (b, 1)))
         assert np.all(val == np.float32(0.25 * d))
+
+
+@pytest.mark.parametrize("V,d,batch,k", [
+    (8192, 64, 256, 1),        # the smallest batch and vocabulary of the filtered GEMM, one K-block
+    (20011, 200, 257, 8),      # a group of one query, a ragged last K-block, every 64th row
+    (20011, 512, 300, 9),      # every 32nd row
+    (30000, 256, 513, 64),     # two blocks, the second of one query
+    (20011, 128, 260, 65),     # every 8th row
+    (8193, 320, 256, 128),     # the largest k, a one-row last tile
+])
+def test_many_queries(vie, V, d, batch, k):
+    """Batches of 256 queries or more: a sample of the rows bounds each query's
+    k-th logit, the logits above it are gathered and ranked."""
+    W, h = workload(V, d, batch, seed=V + batch + k)
+    assert_parity(vie, W, h, k, reps=2)
+
+
+@pytest.mark.parametrize("k", [1, 50])
+def test_many_queries_whose_candidates_overflow(vie, k):
+    """Rows the sample takes (every 64th, hence every 16th) are zero, so every
+    positive logit is a candidate: ~10000 of them, more than are kept, and the
+    query is recomputed; and a zero query, whose logits all tie."""
+    V, d, batch = 20011, 128, 256
+    W, h = workload(V, d, batch, seed=5)
+    W[::16] = 0
+    h[3] = 0.0
+    idx, _, _ = assert_parity(vie, W, h, k)
+    np.testing.assert_array_equal(idx[3], np.arange(k))
