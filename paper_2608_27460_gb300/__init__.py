@@ -83,6 +83,8 @@ def load(path: str | None = None, build_if_missing: bool = True):
     """Load libviehead.so (building it in-tree first if it is missing or
     older than its sources).  Raises if that is impossible."""
     global _lib
+    if _lib is not None and path is None:  # every call passes here: no lock once loaded
+        return _lib
     with _lock:
         if _lib is not None and path is None:
             return _lib
@@ -306,11 +308,26 @@ def check(status: int) -> None:
 
 # ---- torch convenience layer ----------------------------------------------
 
+_current_stream = None
+
+
 def _stream_ptr(stream) -> int:
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+    """The cudaStream_t of `stream`, or of the current stream.  (Building a
+    torch.cuda.Stream object to ask it for its handle was a third of the host
+    time of a small call.)"""
+    global _current_stream
+    if stream is not None:
+        return int(stream.cuda_stream)
+    if _current_stream is None:
+        import torch
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        device = getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and device is not None:
+            torch.cuda.init()
+            _current_stream = lambda: raw(device())  # noqa: E731
+        else:
+            _current_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+    return _current_stream()
 
 
 class Head:
