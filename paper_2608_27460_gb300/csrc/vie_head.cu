@@ -205,18 +205,20 @@ int sel_cap_launch(int nb, int k) {
 }
 
 // Maxima each CTA of a streaming launch publishes per query for the shared
-// bound: the least number that gives 4k of them over the CTAs, at most 8 (of
+// bound: the least number that gives 3k of them over the CTAs, at most 8 (of
 // 32 rows each; fewer than k: none).  With 2k of them the k-th largest lies far
 // below the k-th of their rows, and the merge of k = 300 over 608 maxima got
 // 2100 keys instead of 900, too many for its shared memory (100003 x 1000, k =
-// 300: 42.5 us against 38.8 with 1216 maxima, b = 4: 54.8 against 49.8).
+// 300: 42.5 us against 38.8 with 1216 maxima, b = 4: 54.8 against 49.8); at
+// k = 200 1216 of them cost more to evaluate than they save over 608 (100003 x
+// 1024, b = 8: 82.5 against 73.9 us).
 // None either if a CTA's whole share fits its buffer (k <= 64: ranking that at
 // the end is cheaper than looking for the bound: 11.6 against 12.4 us at
 // 20011 x 640).
 int bound_blocks_for(int k, int64_t V, int G) {
     if (k <= vie::kFastMaxK && V <= static_cast<int64_t>(vie::kSelCapFast) * G) return 0;
     int b = 1;
-    while (b < 8 && b * G < 4 * k) b <<= 1;
+    while (b < 8 && b * G < 3 * k) b <<= 1;
     return b * G >= k && b * G <= vie::kBoundMax ? b : 0;
 }
 
