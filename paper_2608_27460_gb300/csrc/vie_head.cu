@@ -674,7 +674,7 @@ static vie_status run_topk_tc(const char *fn, vie_head *head, const float *h, in
         cudaError_t e = cudaSuccess;
         if (hres_bytes == 0)
             e = q8 ? vie::launch_prep_queries_e4m3(hq, nq, nqt, head->d, head->d_pad, head->hB, head->qscale, s)
-                   : vie::launch_prep_queries(hq, nq, head->d, head->d_pad, 2 * nqt, head->hB, head->num_sms, s);
+                   : vie::launch_prep_queries(hq, nq, head->d, head->d_pad, 2 * nqt, head->hB, s);
         if (e != cudaSuccess) return fail_cuda(e, fn);
         vie::TcParams p;
         p.V = head->V;
@@ -733,8 +733,7 @@ static vie_status run_topk_many(const char *fn, vie_head *head, const float *h, 
         p.cand = head->cand;
         p.count = count;
         p.err = head->words + 1;
-        cudaError_t e = vie::launch_prep_queries(hq, nq, head->d, head->d_pad, groups * 2 * vie::kMnGroup, head->hB,
-                                                 head->num_sms, s);
+        cudaError_t e = vie::launch_prep_queries(hq, nq, head->d, head->d_pad, groups * 2 * vie::kMnGroup, head->hB, s);
         p.rows = rows;
         p.sample = sample;
         p.sample_pitch = pitch;

@@ -85,6 +85,6 @@ cudaError_t launch_prep_queries_e4m3(const float *h, int nq, int nq_tmpl, int d,
 
 // hi/lo bf16 query matrix [n_rows][d_pad] for the tensor-core kernel.
 cudaError_t launch_prep_queries(const float *h, int nq, int d, int d_pad, int n_rows, void *hB,
-                                int sms, cudaStream_t stream);
+                                cudaStream_t stream);
 
 }  // namespace vie

@@ -231,20 +231,100 @@ struct SampleKeys {
 
 }  // namespace
 
-// One CTA per query slot of the block: tau[q] = a key with exactly k sampled
+// One CTA per query slot of the block: tau[q] = a key with at least k sampled
 // keys at or above it, tau_v[q] its logit (+inf for slots without a query, so
-// that none of their logits pass), count[q] = 0.
-__global__ void __launch_bounds__(256) many_tau_kernel(const float *__restrict__ sample, int64_t pitch, int rows,
-                                                       uint32_t stride, int nq, int k, uint64_t *tau, float *tau_v,
-                                                       uint32_t *count) {
-    __shared__ uint32_t hist[256];
+// that none of their logits pass), count[q] = 0.  The sampled logits are read
+// once, into registers; a histogram over the upper half of their range gives
+// the bin of the k-th largest, and the smallest logit of that bin and those
+// above it is the bound.  Where that bin holds many keys (ties, outliers), or
+// the sample more than the registers, a radix select finds the exact k-th key
+// (13.3 us per 512 queries of 2374 sampled rows).
+constexpr int kTauThreads = 512;
+template <int PER>
+__global__ void __launch_bounds__(kTauThreads, PER <= 8 ? 3 : 1) many_tau_kernel(const float *__restrict__ sample, int64_t pitch, int rows,
+                                                               uint32_t stride, int nq, int k, uint64_t *tau, float *tau_v,
+                                                               uint32_t *count) {
+    constexpr int kBins = 1024, kSlack = 4;
+    __shared__ uint32_t hist[kBins];
+    __shared__ uint32_t range[4];  // lowest, highest ordered logit, the k-th largest's bin (+ 1; 0: crowded), bound
     __shared__ MiscSmem ms;
     griddep_launch_dependents();
+    const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) {
+        range[0] = 0xFFFFFFFFu;
+        range[1] = 0u;
+        range[2] = 0u;
+        range[3] = 0xFFFFFFFFu;
+    }
+    for (int i = tid; i < kBins; i += kTauThreads) hist[i] = 0;
     griddep_wait();
-    const int q = blockIdx.x;
     uint64_t t = ~0ull;
-    if (q < nq) t = block_radix_threshold(SampleKeys{sample + q * pitch, stride}, rows, k, 1, hist, &ms);
-    if (threadIdx.x == 0) {
+    if (q < nq) {  // (the whole CTA)
+        const float *z = sample + q * pitch;
+        t = 0;
+        if (rows <= PER * kTauThreads) {
+            uint32_t v[PER], lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) v[j] = tid + j * kTauThreads < rows ? order_f32(z[tid + j * kTauThreads]) : 0u;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                hi = max(hi, v[j]);
+                if (tid + j * kTauThreads < rows) lo = min(lo, v[j]);
+            }
+            lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+            hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+            __syncthreads();
+            if (lane == 0) {
+                atomicMin(&range[0], lo);
+                atomicMax(&range[1], hi);
+            }
+            __syncthreads();
+            // equal bins of the upper half of the logits' range
+            const float top = unorder_f32(range[1]), mid = 0.5f * unorder_f32(range[0]) + 0.5f * top;
+            const float scale = top > mid ? kBins / (top - mid) : 0.0f;
+            int bin[PER];
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                const float x = unorder_f32(v[j]);
+                bin[j] = tid + j * kTauThreads < rows && x >= mid ? min(kBins - 1, static_cast<int>((x - mid) * scale)) : -1;
+                if (bin[j] >= 0) atomicAdd(&hist[bin[j]], 1u);
+            }
+            __syncthreads();
+            if (tid < 32) {  // lane l: bins kBins - 1 - 32 l downwards (read rotated: distinct banks)
+                const int b0 = kBins - 32 - 32 * lane;
+                uint32_t local = 0;
+                for (int j = 0; j < 32; ++j) local += hist[b0 + ((j + lane) & 31)];
+                uint32_t incl = local;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                    if (lane >= o) incl += x;
+                }
+                uint32_t run = incl - local;
+                const uint32_t uk = static_cast<uint32_t>(k);
+                if (run < uk && uk <= incl) {
+                    int b = b0 + 31;
+                    while (run + hist[b] < uk) run += hist[b--];
+                    if (run + hist[b] <= uk + uk / kSlack + kSlack) range[2] = static_cast<uint32_t>(b) + 1u;
+                }
+            }
+            __syncthreads();
+            if (range[2] != 0) {  // the smallest logit of that bin and those above
+                const int b = static_cast<int>(range[2]) - 1;
+                lo = 0xFFFFFFFFu;
+#pragma unroll
+                for (int j = 0; j < PER; ++j)
+                    if (bin[j] >= b) lo = min(lo, v[j]);
+                lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+                if (lane == 0) atomicMin(&range[3], lo);
+                __syncthreads();
+                t = static_cast<uint64_t>(range[3]) << 32;
+            }
+        }
+        __syncthreads();
+        if (t == 0) t = block_radix_threshold(SampleKeys{z, stride}, rows, k, 1, hist, &ms);
+    }
+    if (tid == 0) {
         const uint32_t hi = static_cast<uint32_t>(t >> 32);
         tau[q] = t;
         // (below order_f32(-FLT_MAX) there are only -inf and NaN patterns)
@@ -352,7 +432,8 @@ cudaError_t launch_tc_many(const CUtensorMap &mapW, const CUtensorMap &mapH, con
 
 cudaError_t launch_many_tau(const float *sample, int64_t pitch, int rows, int stride, int nq, int slots, int k,
                             uint64_t *tau, float *tau_v, uint32_t *count, cudaStream_t stream) {
-    return launch_pdl(many_tau_kernel, dim3(static_cast<unsigned>(slots)), dim3(256), 0, stream, sample, pitch, rows,
+    const auto kern = rows <= 8 * kTauThreads ? many_tau_kernel<8> : many_tau_kernel<32>;
+    return launch_pdl(kern, dim3(static_cast<unsigned>(slots)), dim3(kTauThreads), 0, stream, sample, pitch, rows,
                       static_cast<uint32_t>(stride), nq, k, tau, tau_v, count);
 }
 

@@ -15,8 +15,8 @@
 // a key (logit, then row), so neither ties nor clusters of neighbouring rows
 // make many candidates; a list that overflows all the same (kMnCap) is
 // recomputed row by row by its query's CTA.  20000 queries, 151936 x 1024,
-// k = 2: 22.0 ms in passes of 64 queries, 9.2 ms here (per 512 queries: main
-// 191 us, 1.67 PFLOP/s; the other four launches 41 us).
+// k = 2: 22.0 ms in passes of 64 queries, 9.1 ms here (per 512 queries: main
+// 194 us, 1.64 PFLOP/s; the other four launches ~30 us).
 //
 // The GEMM runs on CTA pairs (tcgen05 cta_group::2): M = 256 rows of W, half
 // per CTA, times N = 256 columns, 128 queries as hi and lo. Each CTA stages its

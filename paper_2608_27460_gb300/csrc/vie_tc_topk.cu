@@ -8,20 +8,27 @@
 namespace vie {
 
 // hB[n_rows][d_pad] bf16: row 2q = rn(h_q), row 2q+1 = rn(h_q - rn(h_q)),
-// rows of absent queries and columns >= d are zero.
-__global__ void prep_queries_kernel(const float *__restrict__ h, int nq, int d, int d_pad,
-                                    int n_rows, __nv_bfloat16 *__restrict__ hB) {
+// rows of absent queries and columns >= d are zero.  Two columns of both rows
+// per thread (grid (ceil(d_pad / kPrepCols), n_rows / 2)): no divisions and one
+// round trip (512 queries of 1024 columns: 7.7 us with a 64-bit division per
+// element, 3.6 us).
+constexpr int kPrepThreads = 256, kPrepCols = 2 * kPrepThreads;
+__global__ void __launch_bounds__(kPrepThreads) prep_queries_kernel(const float *__restrict__ h, int nq, int d,
+                                                                    int d_pad, __nv_bfloat16 *__restrict__ hB) {
     griddep_launch_dependents();  // the projection kernel may start its prologue now
     griddep_wait();  // h comes from the kernel before this one, which may still read hB
-    const int64_t n = static_cast<int64_t>(n_rows) * d_pad;
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int r = static_cast<int>(i / d_pad), j = static_cast<int>(i - static_cast<int64_t>(r) * d_pad);
-        const int q = r >> 1;
-        const float x = (q < nq && j < d) ? h[static_cast<int64_t>(q) * d + j] : 0.0f;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-        hB[i] = (r & 1) ? __float2bfloat16_rn(x - __bfloat162float(hi)) : hi;
-    }
+    const int q = blockIdx.y, j = blockIdx.x * kPrepCols + 2 * static_cast<int>(threadIdx.x);
+    if (j >= d_pad) return;  // (d_pad is even)
+    const float *hq = h + static_cast<int64_t>(q) * d;
+    const float x0 = q < nq && j < d ? hq[j] : 0.0f, x1 = q < nq && j + 1 < d ? hq[j + 1] : 0.0f;
+    __nv_bfloat162 hi, lo;
+    hi.x = __float2bfloat16_rn(x0);
+    hi.y = __float2bfloat16_rn(x1);
+    lo.x = __float2bfloat16_rn(x0 - __bfloat162float(hi.x));
+    lo.y = __float2bfloat16_rn(x1 - __bfloat162float(hi.y));
+    __nv_bfloat16 *row = hB + static_cast<int64_t>(2 * q) * d_pad + j;
+    *reinterpret_cast<__nv_bfloat162 *>(row) = hi;
+    *reinterpret_cast<__nv_bfloat162 *>(row + d_pad) = lo;
 }
 
 template <int NQ, bool Q8>
@@ -119,12 +126,10 @@ cudaError_t launch_tc_topk(int nq_tmpl, bool q8, const CUtensorMap &mapW, const 
 }
 
 cudaError_t launch_prep_queries(const float *h, int nq, int d, int d_pad, int n_rows, void *hB,
-                                int sms, cudaStream_t stream) {
-    const int64_t n = static_cast<int64_t>(n_rows) * d_pad;
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 4LL * sms) blocks = 4LL * sms;
-    return launch_pdl(prep_queries_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, stream, h, nq, d,
-                      d_pad, n_rows, static_cast<__nv_bfloat16 *>(hB));
+                                cudaStream_t stream) {
+    const dim3 grid(static_cast<unsigned>((d_pad + kPrepCols - 1) / kPrepCols), static_cast<unsigned>(n_rows / 2));
+    return launch_pdl(prep_queries_kernel, grid, dim3(kPrepThreads), 0, stream, h, nq, d, d_pad,
+                      static_cast<__nv_bfloat16 *>(hB));
 }
 
 }  // namespace vie
