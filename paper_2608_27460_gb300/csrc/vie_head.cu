@@ -651,17 +651,20 @@ static vie_status run_topk_tc(const char *fn, vie_head *head, const float *h, in
                               cudaStream_t s) {
     const bool q8 = head->scale != nullptr;
     const int nqt = tc_group(batch, k, q8);
-    // K-blocks per stage: the most that still leave a ring of two stages
-    // (larger stages beat deeper rings of small ones); the query boxes stay
-    // resident in shared memory when they are small (e4m3 rows)
+    // K-blocks per stage: the most that still leave a ring of three stages
+    // (larger stages beat deeper rings of small ones: every stage costs its
+    // refill ~0.1 us; but with two, one in flight is too little: 128256 x 3072,
+    // b = 16: 125.0 us with 2 x 4 K-blocks, 122.0 with 3 x 3; b = 64: 137.4 with
+    // 2 x 3, 134.8 with 3 x 2), else of two; the query boxes stay resident in
+    // shared memory when they are small (e4m3 rows)
     int stages = 0, kps = 0, slots = 0;
     uint32_t smem = 0;
     int kps_max = opt(VIE_OPT_TC_KPS);
     kps_max = kps_max > vie::kTcMaxKPS ? vie::kTcMaxKPS : kps_max;
     const int hres_bytes = tc_hres(head, nqt);
-    for (int c = kps_max; c >= 1 && kps == 0; --c) {
-        if (vie::tc_shape(nqt, q8, c, hres_bytes, &stages, &slots, &smem)) kps = c;
-    }
+    for (int least = 3; least >= 2 && kps == 0; --least)
+        for (int c = kps_max; c >= 1 && kps == 0; --c)
+            if (vie::tc_shape(nqt, q8, c, hres_bytes, &stages, &slots, &smem) && stages >= least) kps = c;
     if (kps == 0) return fail(VIE_ERR_UNSUPPORTED, "%s: no tensor-core layout", fn);
     const int tile_rows = vie::tc_tile_rows(nqt, q8);
     const int n_tiles = static_cast<int>((head->V + tile_rows - 1) / tile_rows);

@@ -449,7 +449,11 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
             // With static tiles to issue first, the wait has long been over.
             if (Ns == 0) griddep_wait();
             uint32_t draw = (Ns == 0) ? atomic_add_relaxed_gpu(p.next_tile, 1u) : 0u;
-            int it = 0, issued = 0;
+            // ring position s and the parity of its current use, kept by counting
+            // (a division by the run-time depth per stage is a dependent chain in
+            // front of every refill)
+            int s = 0, issued = 0;
+            uint32_t ph = 0;
             bool ok = true;
             for (int ti = 0; ok; ++ti) {
                 int tile;
@@ -464,9 +468,8 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                     draw = atomic_add_relaxed_gpu(p.next_tile, 1u);
                 }
                 const int nst = tile < 0 ? 1 : n_st;
-                for (int st_i = 0; st_i < nst; ++st_i, ++it) {
-                    const int s = it % S, u = it / S;
-                    if (it >= S && !mbar_wait(&empty[s], (u - 1) & 1, abort_flag)) {
+                for (int st_i = 0; st_i < nst; ++st_i) {
+                    if (issued >= S && !mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
                         ok = false;
                         break;
                     }
@@ -484,12 +487,16 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                             tma_load_2d(st + i * Sh::kStageA + h * Sh::kHalfA, &mapW, (kb0 + i) * KB,
                                         tile * TR + h * kTcTile, &full[s], pol);
                     if (!hres) {
-                        if (it == 0) griddep_wait();  // the query matrix comes from the prep kernel
+                        if (issued == 0) griddep_wait();  // the query matrix comes from the prep kernel
                         for (int i = 0; i < nin; ++i)
                             tma_load_2d(st + KPS * Sh::kStageA + i * Sh::kStageB, &mapH,
                                         (kb0 + i) * KB, 0, &full[s], pol);
                     }
-                    issued = it + 1;
+                    ++issued;
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
                 if (tile < 0) break;
             }
@@ -508,16 +515,16 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
             constexpr uint32_t idesc = Q8 ? umma_idesc_e4m3_f32(kTcTile, N) : umma_idesc_bf16_f32(kTcTile, N);
-            int it = 0;
+            int s = 0;
+            uint32_t ph = 0;
             bool ok = true;
             for (int ti = 0; ok; ++ti) {
                 const int b = ti & 1, ub = ti >> 1;
-                const int s0 = it % S, u0 = it / S;
-                if (!mbar_wait(&full[s0], u0 & 1, abort_flag)) {
+                if (!mbar_wait(&full[s], ph, abort_flag)) {
                     ok = false;
                     break;
                 }
-                const int tile = mc->stage_tile[s0];
+                const int tile = mc->stage_tile[s];
                 if (ti >= 2 && !mbar_wait(&tempty[b], (ub - 1) & 1, abort_flag)) {
                     ok = false;
                     break;
@@ -531,9 +538,8 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                 }
                 mc->buf_tile[b] = tile;
                 const uint32_t d = tmem + static_cast<uint32_t>(b * Sh::kAccCols);
-                for (int st_i = 0; st_i < n_st; ++st_i, ++it) {
-                    const int s = it % S, u = it / S;
-                    if (st_i > 0 && !mbar_wait(&full[s], u & 1, abort_flag)) {
+                for (int st_i = 0; st_i < n_st; ++st_i) {
+                    if (st_i > 0 && !mbar_wait(&full[s], ph, abort_flag)) {
                         ok = false;
                         break;
                     }
@@ -558,6 +564,10 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                         }
                     }
                     umma_commit(&empty[s]);
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
                 if (!ok) break;
                 umma_commit(&tfull[b]);
