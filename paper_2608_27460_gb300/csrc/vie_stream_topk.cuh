@@ -1388,6 +1388,8 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
             if (Ns == 0) griddep_wait();
             uint32_t draw = (Ns == 0 && pool) ? atomic_add_relaxed_gpu(p.next_chunk, 1u) : 0u;
             int issued = 0;
+            int s = 0;  // ring position and the parity of its use, kept by counting
+            uint32_t ph = 0;
             bool ok = true;
             for (int t = 0;; ++t) {
                 int64_t row0;
@@ -1399,8 +1401,7 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
                 } else {
                     row0 = -1;
                 }
-                const int s = t % S, u = t / S;
-                if (t >= S && !mbar_wait(&empty[s], (u - 1) & 1, abort_flag)) {
+                if (t >= S && !mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
                     ok = false;
                     break;
                 }
@@ -1414,6 +1415,10 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
                 mbar_arrive_expect_tx(&full[s], bytes);
                 bulk_g2s(ring + s * stage_bytes, W + row0 * row_bytes, bytes, &full[s], pol);
                 issued = t + 1;
+                if (++s == S) {
+                    s = 0;
+                    ph ^= 1u;
+                }
                 if (t + 1 == Ns) griddep_wait();
                 if (t + 1 >= Ns && pool) draw = atomic_add_relaxed_gpu(p.next_chunk, 1u);
             }
@@ -1600,10 +1605,11 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
         } else {
             // ---------------- projection ----------------
             const int w = warp - 1 - NS;
-            int t = 0;
+            int t = 0, s_next = 0;
+            uint32_t ph = 0;
             for (;; ++t) {
-                const int s = t % S, u = t / S;
-                if (!mbar_wait(&full[s], u & 1, abort_flag)) {
+                const int s = s_next;
+                if (!mbar_wait(&full[s], ph, abort_flag)) {
                     if (lane == 0) {
                         atomicOr(p.err, kErrWaitTimeout);
                         ms->abort = 1;
@@ -1612,6 +1618,10 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
                 }
                 const int chunk = ms->chunk_w[s];
                 if (chunk < 0) break;
+                if (++s_next == S) {
+                    s_next = 0;
+                    ph ^= 1u;
+                }
                 const int64_t row0 = chunk;
                 const int rows = stage_rows(row0, pool_row0, RS, RSH, p.V);
                 const unsigned char *stage = ring + s * stage_bytes;
