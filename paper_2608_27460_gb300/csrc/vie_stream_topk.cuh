@@ -128,6 +128,7 @@ struct StreamTopkParams {
     int32_t *out_idx;        // [nq, k]
     float *out_logits;       // [nq, k]
     float *sparse;           // [nq, V] fp32 or nullptr
+    int32_t reverse;         // 1: W's chunks are taken from the last to the first (pool_rows == rows_per_stage)
     int32_t pdl;             // 1: W is constant, so the launch may overlap the kernel before it
 };
 
@@ -1379,6 +1380,7 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
             const uint64_t pol = l2_evict_first_policy();
             const unsigned char *W = reinterpret_cast<const unsigned char *>(p.W);
             const int Ns = p.static_chunks;
+            const int64_t last_row0 = (p.V - 1) / RS * RS;  // the last chunk's first row
             // the early merger (CTA 0) streams its round-robin chunks only
             const bool pool = !(p.early && cta == 0);
             // The pool counter is re-armed by the previous launch on the
@@ -1401,6 +1403,7 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
                 } else {
                     row0 = -1;
                 }
+                if (p.reverse && row0 >= 0) row0 = last_row0 - row0;
                 if (t >= S && !mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
                     ok = false;
                     break;
