@@ -1383,10 +1383,14 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
             const int64_t last_row0 = (p.V - 1) / RS * RS;  // the last chunk's first row
             // the early merger (CTA 0) streams its round-robin chunks only
             const bool pool = !(p.early && cta == 0);
-            // The pool counter is re-armed by the previous launch on the
-            // handle, which this one may overlap: the first draw waits for it
-            // (with round-robin chunks to issue first, long over by then).
-            // The draw itself is issued early so its latency is hidden.
+            // One stage is requested at once, the others when the kernel before
+            // this one has finished: a whole ring per SM, 29 MB, queues up in
+            // front of that kernel's merge, whose polls and list reads then take
+            // 4 us instead of 1.5 (151936 x 1024, b = 1, back to back: 48.6 us
+            // with the whole ring, 47.5 with one stage; two stages are no better
+            // than the ring).  The pool counter, re-armed at that kernel's end,
+            // is drawn from after the same wait, and early, so that the draw's
+            // latency is hidden.
             if (Ns == 0) griddep_wait();
             uint32_t draw = (Ns == 0 && pool) ? atomic_add_relaxed_gpu(p.next_chunk, 1u) : 0u;
             int issued = 0;
@@ -1422,7 +1426,7 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
                     s = 0;
                     ph ^= 1u;
                 }
-                if (t + 1 == Ns) griddep_wait();
+                if (t == 0) griddep_wait();
                 if (t + 1 >= Ns && pool) draw = atomic_add_relaxed_gpu(p.next_chunk, 1u);
             }
             if (!ok) {
