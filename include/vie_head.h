@@ -375,7 +375,8 @@ vie_status vie_scatter_sparse_logits(const int32_t *idx, const float *logits, in
  *         while cap * c * 8 > 32768, where c = max(256, 2k rounded up to a
  *         multiple of 64) is the candidate buffer of one query.
  * Scratch: one 1 MiB array per device (every GPU that loads the library keeps
- * it until the process exits), of which the first 256 bytes hold counters.
+ * it until the process exits), of which the first 256 bytes hold counters, and
+ * 80 KiB behind it for the bounds that the CTAs of a launch share.
  * A call needs
  *   8 * (round_up_even(slots * ctas * k) + slots * ctas * 8)
  * bytes of the rest, where ctas = min(SM count, ceil(V / 64), 1024) and
@@ -383,8 +384,8 @@ vie_status vie_scatter_sparse_logits(const int32_t *idx, const float *logits, in
  * requests return VIE_ERR_UNSUPPORTED with the sizes in the message.  Groups
  * of one call run one after the other on `stream` and reuse the same lists
  * (the kernel re-arms its counters at the end of each launch).  The call clears
- * the counters at the start of the array with cudaMemsetAsync on `stream`
- * and allocates nothing (no cudaMalloc, no cudaFree, no allocating library
+ * the counters and the bounds with cudaMemsetAsync on `stream` and allocates
+ * nothing (no cudaMalloc, no cudaFree, no allocating library
  * routine).
  * The first call on a device looks up the array's device address with
  * cudaGetSymbolAddress (once per device); make that first call before any

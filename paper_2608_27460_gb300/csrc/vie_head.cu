@@ -79,7 +79,7 @@ struct vie_head {
     uint64_t *gmax;     // [G * kBoundWords] maxima behind the shared bounds (tagged words), in cand's allocation
     int64_t scratch_bytes;
     // tensor-core path (batches): hi/lo bf16 query matrix and TMA descriptors
-    void *hB;             // [kHRows][d_pad] bf16, or e4m3 query pieces [4 NQ][d_pad]
+    void *hB;             // [kHRows][d_pad] bf16, or e4m3 query pieces [4 NQ][d_pad]; in cand's allocation
     float *qscale;        // e4m3 heads: [32][kQ8Pieces] piece scales of the query group
     bool tc_ready;
     CUtensorMap mapW;     // W as [V][d_pad], box 128 rows x 128 bytes, 128-byte swizzle
@@ -477,14 +477,17 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
     hd->scratch_bytes = static_cast<int64_t>(cbytes + gbytes + mbytes + kNumWords * sizeof(uint32_t));
     e = cudaMalloc(&hd->W, wbytes);
     if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->scale, static_cast<size_t>(V) * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&hd->cand, cbytes + gbytes + mbytes);
-    // bounds of no launch (tag 0); empty lists until written
-    if (e == cudaSuccess) e = cudaMemset(hd->cand, 0, cbytes + gbytes + mbytes);
-    if (e == cudaSuccess) hd->gmax = hd->cand + cbytes / sizeof(uint64_t);
+    // one allocation and one clear: tagged words of no launch (tag 0), empty
+    // lists until written, zero query rows
+    const size_t hoff = (cbytes + gbytes + mbytes + 255) & ~static_cast<size_t>(255);
+    const size_t hbytes = static_cast<size_t>(e4m3 ? vie::kTcHRows : kHRows) * hd->d_pad * 2;
+    if (e == cudaSuccess) e = cudaMalloc(&hd->cand, hoff + hbytes);
+    if (e == cudaSuccess) e = cudaMemset(hd->cand, 0, hoff + hbytes);
+    if (e == cudaSuccess) {
+        hd->gmax = hd->cand + cbytes / sizeof(uint64_t);
+        hd->hB = reinterpret_cast<unsigned char *>(hd->cand) + hoff;
+    }
     if (e == cudaSuccess) e = cudaMalloc(&hd->words, kNumWords * sizeof(uint32_t));
-    if (e == cudaSuccess)
-        e = cudaMalloc(&hd->hB, static_cast<size_t>(e4m3 ? vie::kTcHRows : kHRows) * hd->d_pad * 2);
-    if (e == cudaSuccess) e = cudaMemset(hd->hB, 0, static_cast<size_t>(vie::kTcHRows) * hd->d_pad * 2);
     if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->qscale, 32 * vie::kQ8Pieces * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(hd->words, 0, kNumWords * sizeof(uint32_t));
     if (e == cudaSuccess && e4m3) {
@@ -509,7 +512,6 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
         cudaFree(hd->scale);
         cudaFree(hd->cand);
         cudaFree(hd->words);
-        cudaFree(hd->hB);
         cudaFree(hd->qscale);
         delete hd;
         return st;
@@ -567,7 +569,6 @@ vie_status vie_head_destroy(vie_head *head) {
     cudaFree(head->scale);
     cudaFree(head->cand);
     cudaFree(head->words);
-    cudaFree(head->hB);
     cudaFree(head->qscale);
     cudaFree(head->stage_h);
     cudaFree(head->stage_idx);

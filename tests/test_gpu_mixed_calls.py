@@ -52,3 +52,28 @@ def test_mixed_paths_back_to_back(vie, storage):
     for (b, k), (ai, av) in zip(CALLS, alone):
         for r in range(b):
             assert not check_topk(ai[r], av[r], z[r], k), (b, k, r)
+
+
+@pytest.mark.parametrize("storage,batch,k", [("bf16", 1, 50), ("bf16", 1, 300), ("bf16", 4, 50), ("bf16", 5, 300),
+                                             ("bf16", 300, 2), ("e4m3", 1, 50), ("e4m3", 12, 50)])
+def test_queries_written_just_before_each_call(vie, storage, batch, k):
+    """Launches overlap the kernels before them on the stream: each step's
+    queries are written into the same buffer right before its call and the
+    next step's right behind it, with nothing waiting in between."""
+    import torch
+    V, d, steps = 30011, 512, 12
+    W, h = workload(V, d, steps * batch, seed=61)
+    src = torch.from_numpy(h).cuda().view(steps, batch, d)
+    with vie.Head(to_device_bits(W), storage=storage) as head:
+        alone = [tuple(t.clone() for t in head.topk(src[s].contiguous(), k)) for s in range(steps)]
+        torch.cuda.synchronize()
+        buf = torch.empty((batch, d), device="cuda")
+        outs = []
+        for s in range(steps):
+            buf.copy_(src[s])
+            outs.append(head.topk(buf, k))
+        torch.cuda.synchronize()
+        assert head.device_status() == vie.VIE_OK
+    for (ai, av), (i, v) in zip(alone, outs):
+        np.testing.assert_array_equal(i.cpu().numpy(), ai.cpu().numpy())
+        np.testing.assert_array_equal(v.cpu().numpy().view(np.uint32), av.cpu().numpy().view(np.uint32))

@@ -105,3 +105,30 @@ def test_many_queries_whose_candidates_overflow(vie, k):
     h[3] = 0.0
     idx, _, _ = assert_parity(vie, W, h, k)
     np.testing.assert_array_equal(idx[3], np.arange(k))
+
+
+def test_many_queries_sparse_and_captured(vie):
+    """The sparse rows of a filtered-GEMM call equal the scatter of its own
+    top-k, and replaying the captured call gives the eager bits."""
+    import torch
+    V, d, batch, k = 8300, 128, 260, 50
+    W, h = workload(V, d, batch, seed=77)
+    hd = torch.from_numpy(h).cuda()
+    with vie.Head(to_device_bits(W)) as head:
+        assert head.plan(batch, k).launches == 5
+        ei, ev, es = head.topk_sparse(hd, k)
+        want = head.sparse_logits(ei, ev)
+        oi, ov, osp = torch.empty_like(ei), torch.empty_like(ev), torch.empty_like(es)
+        cap = torch.cuda.Stream()
+        cap.wait_stream(torch.cuda.current_stream())
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(cap), torch.cuda.graph(g, stream=cap):
+            head.topk_sparse(hd, k, out_idx=oi, out_logits=ov, out_sparse=osp, stream=cap)
+        torch.cuda.current_stream().wait_stream(cap)
+        for _ in range(2):
+            osp.zero_()
+            g.replay()
+        torch.cuda.synchronize()
+        assert head.device_status() == vie.VIE_OK
+    for a, b in ((es, want), (oi, ei), (ov, ev), (osp, es)):
+        np.testing.assert_array_equal(a.cpu().numpy().view(np.uint32), b.cpu().numpy().view(np.uint32))
