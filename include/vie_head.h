@@ -131,7 +131,9 @@ vie_status vie_head_destroy(vie_head *head);
 /* Fills *props (host) with the handle's facts. */
 vie_status vie_head_get_props(const vie_head *head, vie_head_props *props);
 
-/* How a vie_head_topk / vie_head_topk_sparse call of this size runs. */
+/* How a vie_head_topk / vie_head_topk_sparse call of this size runs.  (bf16
+ * batches of 256 queries or more with k <= 128 run as a filtered GEMM on the
+ * tensor cores: groups of 128 queries, five launches per block of up to 512.) */
 typedef struct {
     int32_t path;     /* 0: streaming CUDA-core kernel, 1: tensor-core kernel  */
     int32_t groups;   /* query groups, one pass over W_out each               */

@@ -24,7 +24,7 @@
 //              are left.  For k <= 64 those go into a sorted list spread over
 //              the warp's registers (an insertion is ~0.14 us), which is final
 //              when the stream ends (100003 x 1000, b = 1: 39.8 -> 33.7 us at
-//              k = 50, 49.3 -> 42.5 us at k = 300);
+//              k = 50, 49.3 -> 38.8 us at k = 300);
 //   the next 8 warps  projection: warp w owns rows w, w+8, .. (at most R) of
 //              each stage and every lane a strided set of 16-byte column
 //              chunks; bf16 -> fp32 widening, fp32 FMA against h (staged in
@@ -33,22 +33,24 @@
 //              shared-memory read retires; the warp-shuffle sums then go to
 //              a separate, deeper score ring.
 // The full logit vector never leaves the chip.  Afterwards each CTA writes
-// its sorted top-k list to scratch and takes a ticket (an acq_rel atomic, no
-// full fences); the CTA that draws the last ticket copies every list into
-// shared memory in one pass (when they fit) and merges them:
+// its list to scratch, and the lists are merged in the same launch.  The full
+// merge of sorted lists:
 //   1. tau* = k-th largest key among the first J = ceil(k/G) entries of all
 //      lists (a lower bound of the true k-th key: k keys are >= it);
 //   2. every list contributes its prefix of keys >= tau*;
-//   3. exact top-k of those candidates (rank counting, or radix select when
-//      there are many), written best first.
+//   3. exact top-k of those candidates (a counting sort, or a radix select
+//      first when there are many), written best first.
+// Where nothing is published (the no-alloc entry point), the CTA that draws
+// the last ticket (an acq_rel atomic, no full fences) runs it.
 // Single-query launches with k <= 64 merge early instead: CTA 0 streams only
 // its round-robin chunks (never the pool), so it finishes first, and then
 // merges the CTAs' lists as they are published (merge_published: a release
 // store of the launch's epoch per CTA, polled with acquire loads, the lists'
 // first keys gathered in shared memory as they come); after the last list
 // only one poll, one load and the fast merge over those keys remain.
-// Launches of several queries publish their lists the same way; the first
-// CTAs to finish (one per query, round robin) merge them as they arrive.
+// Launches of several queries, or with k > 64, publish their lists the same
+// way; the first CTAs to finish (one per query, round robin) merge them as they
+// arrive (k > 64: merge_published_wide, from the lists' 32 best keys).
 // With a sparse output, every CTA first fills a fixed slice of each output
 // row with -inf; the merging CTA writes the k logits after every CTA has
 // finished (the last ticket, or the last published list), so each fill
