@@ -17,6 +17,7 @@
 
 #include "vie_head.h"
 #include "vie_launch.h"
+#include "vie_plan.h"
 #include "vie_tc_many.cuh"
 #include "vie_tc_topk.cuh"
 
@@ -57,9 +58,6 @@ constexpr int kEpochWord = 4;
 constexpr int kFlagWords = 8;
 constexpr int kCountWords = kFlagWords + vie::kMaxLists;
 constexpr int kNumWords = kCountWords + vie::kTcMaxSelWarps;
-// Words per CTA of the shared bounds' maxima (gmax): 8 queries x 8 on the
-// streaming path, 64 x 1 or 32 x 4 on the tensor-core path.
-constexpr int kBoundWords = 128;
 // Rows of a bf16 head's query matrix: hi and lo of a block of many queries.
 constexpr int kHRows = 2 * vie::kMnBlock;
 static_assert(kHRows >= vie::kTcHRows, "the batched path's query matrix fits");
@@ -76,7 +74,7 @@ struct vie_head {
     float *scale;       // e4m3 heads: fp32 scale per row [V]; nullptr for bf16 heads
     uint64_t *cand;     // [kMaxNB][G][VIE_K_MAX] ranking keys, then [kMaxNB][G][kWideE] heads
     uint32_t *words;    // kNumWords scratch words (see kEpochWord, kFlagWords)
-    uint64_t *gmax;     // [G * kBoundWords] maxima behind the shared bounds (tagged words), in cand's allocation
+    uint64_t *gmax;     // [G * vie::kBoundWords] maxima behind the shared bounds (tagged words), in cand's allocation
     int64_t scratch_bytes;
     // tensor-core path (batches): hi/lo bf16 query matrix and TMA descriptors
     void *hB;             // [kHRows][d_pad] bf16, or e4m3 query pieces [4 NQ][d_pad]; in cand's allocation
@@ -471,7 +469,7 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
     const size_t wbytes = static_cast<size_t>(V) * hd->d_pad * (e4m3 ? 1 : 2);
     const size_t cbytes =
         static_cast<size_t>(kMaxNB) * hd->G * (VIE_K_MAX + vie::kWideE) * sizeof(uint64_t);
-    const size_t gbytes = static_cast<size_t>(hd->G) * kBoundWords * sizeof(uint64_t);
+    const size_t gbytes = static_cast<size_t>(hd->G) * vie::kBoundWords * sizeof(uint64_t);
     const size_t mbytes = static_cast<size_t>(vie::kMnBlock) * (sizeof(uint64_t) + 2 * sizeof(float));
     hd->cand_bytes = cbytes;
     hd->scratch_bytes = static_cast<int64_t>(cbytes + gbytes + mbytes + kNumWords * sizeof(uint32_t));
@@ -698,9 +696,7 @@ static vie_status run_topk_tc(const char *fn, vie_head *head, const float *h, in
         p.flags = head->words + kFlagWords;
         p.counts = head->words + kCountWords;
         p.gmax = head->gmax;
-        // a maximum per tile, or per 32 rows where the CTAs' maxima would be too few for k
-        p.gt_blocks = 2 * k <= head->G ? 1 : 4;
-        if (p.gt_blocks * head->G < k || p.gt_blocks * head->G > vie::kBoundMax) p.gt_blocks = 0;
+        p.gt_blocks = vie::tc_bound_blocks(nqt, k, head->G);
         p.out_idx = out_idx + static_cast<int64_t>(q0) * k;
         p.out_logits = out_logits + static_cast<int64_t>(q0) * k;
         p.sparse = sparse != nullptr ? sparse + static_cast<int64_t>(q0) * head->V : nullptr;
@@ -722,7 +718,7 @@ static vie_status run_topk_many(const char *fn, vie_head *head, const float *h, 
     const int rows = static_cast<int>((head->V + stride - 1) / stride);
     const int64_t pitch = many_pitch(head, k);
     float *sample = reinterpret_cast<float *>(head->cand);  // read for the bounds before candidates replace it
-    uint64_t *tau = head->gmax + static_cast<size_t>(head->G) * kBoundWords;
+    uint64_t *tau = head->gmax + static_cast<size_t>(head->G) * vie::kBoundWords;
     float *tau_v = reinterpret_cast<float *>(tau + vie::kMnBlock);
     uint32_t *count = reinterpret_cast<uint32_t *>(tau_v + vie::kMnBlock);
     for (int q0 = 0; q0 < batch; q0 += block) {

@@ -64,6 +64,7 @@
 #include <type_traits>
 
 #include "vie_device.cuh"
+#include "vie_plan.h"
 
 namespace vie {
 
@@ -86,7 +87,6 @@ constexpr int kFastE = 8;              // fast merge: entries read per list (eve
 constexpr int kFastMaxK = 64;          // fast merge: largest k
 constexpr int kWideE = 32;             // published wide lists: sorted keys per list in the heads area
 constexpr int kSelCapFast = 256;       // candidate buffer keys per query, k <= kFastMaxK
-constexpr int kBoundMax = 1280;        // maxima behind a shared bound, at most
 constexpr int kBoundBlocks = 4;        // row blocks of 32 a CTA's shared maxima cover, at least
 constexpr int kSelRun = 128;           // keys of one sorted run (a warp's registers)
 

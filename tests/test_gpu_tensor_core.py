@@ -5,6 +5,8 @@ settle from the lists' heads and hands to the full merge."""
 import numpy as np
 import pytest
 
+import oracle
+from acceptance import check_topk
 from gpu_cases import assert_parity, run_head, to_device_bits, workload
 from paper_2608_27460_gb300 import synth
 
@@ -45,6 +47,32 @@ def test_plan_selects_paths(vie):
 def test_tensor_core_parity(vie, V, d, batch, k):
     W, h = workload(V, d, batch, seed=V + batch + k)
     assert_parity(vie, W, h, k, reps=2)
+
+
+# fewer CTAs than 2 k (64 rows each): every CTA publishes four maxima per query
+@pytest.mark.parametrize("storage", ["bf16", "e4m3"])
+@pytest.mark.parametrize("V,k", [(1000, 20), (1000, 50), (1100, 64), (2500, 20), (2500, 50), (2500, 64),
+                                 (5000, 50), (6000, 50), (8127, 64)])
+@pytest.mark.parametrize("d", [64, 1024, 3072])
+def test_bound_words_of_small_vocabularies(vie, storage, V, d, k):
+    """The words of the CTAs' shared bound and the query matrix lie next to
+    each other: groups of 8 to 64 queries, repeated without waiting, give the
+    oracle's top-k and every launch the same bits."""
+    import torch
+    W, h = workload(V, d, 100, seed=V + d + k)
+    z = oracle.logits(W, h) if storage == "bf16" else oracle.logits_e4m3(*oracle.quantize_e4m3(W), h)
+    hd = torch.from_numpy(h).cuda()
+    with vie.Head(to_device_bits(W), storage=storage) as head:
+        for b in (8, 32, 33, 64, 100):
+            outs = [head.topk(hd[:b], k) for _ in range(4)]
+            torch.cuda.synchronize()
+            assert head.device_status() == vie.VIE_OK
+            idx, val = (t.cpu().numpy() for t in outs[0])
+            for i, v in outs[1:]:
+                np.testing.assert_array_equal(i.cpu().numpy(), idx)
+                np.testing.assert_array_equal(v.cpu().numpy().view(np.uint32), val.view(np.uint32))
+            for q in range(b):
+                assert not check_topk(idx[q], val[q], z[q], k), (b, q)
 
 
 def _crowded(V, d, batch, rows, seed):

@@ -1,0 +1,40 @@
+"""Launch-planning rules that need no GPU (csrc/vie_plan.h), compiled and
+enumerated here over every shape a call can take."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2608_27460_gb300", "csrc")
+
+
+def run_cpp(tmp_path, body):
+    """Compiles `body` as main() behind vie_plan.h and returns its output lines."""
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no g++")
+    src, exe = tmp_path / "plan.cpp", tmp_path / "plan"
+    src.write_text('#include <cstdio>\n#include <initializer_list>\n#include "vie_plan.h"\nusing namespace vie;\nint main() {\n' + body + "\n}\n")
+    subprocess.run([gxx, "-std=c++17", "-O1", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split("\n")[:-1]
+
+
+def test_shared_bound_words_stay_within_their_room(tmp_path):
+    """A tensor-core launch of `slots` query slots publishes slots * blocks
+    words per CTA; what lies behind the kBoundWords of a handle is the query
+    matrix the same launch reads.  Every tile, k and number of CTAs: 64 slots
+    take k up to 64, the others up to 128.  The bound is used wherever one
+    maximum per CTA gives k of them."""
+    out = run_cpp(tmp_path, """
+    for (int slots : {4, 8, 16, 32, 64})
+        for (int k = 1; k <= (slots == 64 ? 64 : 128); ++k)
+            for (int G = 1; G <= 1024; ++G) {
+                const int b = tc_bound_blocks(slots, k, G);
+                if (b != 0 && b != 1 && b != 4) std::printf("blocks %d %d %d: %d\\n", slots, k, G, b);
+                if (slots * b > kBoundWords) std::printf("words %d %d %d: %d\\n", slots, k, G, b);
+                if (b != 0 && (b * G < k || b * G > kBoundMax)) std::printf("count %d %d %d: %d\\n", slots, k, G, b);
+                if (b == 0 && G >= k) std::printf("unused %d %d %d\\n", slots, k, G);
+            }""")
+    assert not out, out[:10]
