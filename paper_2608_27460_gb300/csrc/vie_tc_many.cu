@@ -103,6 +103,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMnThreads, 1)
     } else if (warp == 1) {
         // ---------------- MMA issuer (the leader's) ----------------
         if (lane == 0 && rank == 0) {
+            griddep_wait();  // the limit of the waits below counts from here, not from a start under an earlier kernel
             constexpr uint32_t idesc = umma_idesc_bf16_f32(kMnRows, 2 * kMnGroup);
             int it = 0, ti = 0;
             bool ok = true;

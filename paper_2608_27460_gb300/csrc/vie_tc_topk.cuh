@@ -469,6 +469,7 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                 }
                 const int nst = tile < 0 ? 1 : n_st;
                 for (int st_i = 0; st_i < nst; ++st_i) {
+                    if (issued == S) griddep_wait();  // as for the MMA issuer's waits
                     if (issued >= S && !mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
                         ok = false;
                         break;
@@ -514,6 +515,7 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
+            griddep_wait();  // the limit of the waits below counts from here, not from a start under an earlier kernel
             constexpr uint32_t idesc = Q8 ? umma_idesc_e4m3_f32(kTcTile, N) : umma_idesc_bf16_f32(kTcTile, N);
             int s = 0;
             uint32_t ph = 0;
@@ -587,8 +589,8 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
         // ---------------- epilogue: TMEM -> logits ----------------
         const int qw = warp & 3;  // TMEM lane quarter this warp may access
         const int row = 32 * qw + lane;
+        griddep_wait();  // the prep kernel wrote the scales; and as for the MMA issuer's waits
         if (Q8 && !hres) {
-            griddep_wait();  // the prep kernel wrote them
             const int e = (warp - 2) * 32 + lane;
             if (e < NQ * kQ8Pieces) qs[e] = p.qscale[e];
             named_barrier_sync(2, 128);  // the four epilogue warps
