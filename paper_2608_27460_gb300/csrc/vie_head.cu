@@ -364,13 +364,8 @@ bool make_map_bf16(CUtensorMap *m, void *base, uint64_t rows, uint64_t cols, uin
 constexpr int kManyMinBatch = 256;
 constexpr int64_t kManyMinRows = 8192;  // a smaller vocabulary's sample bounds too little
 
-// The sample takes every (8 << i)-th row: the widest stride, 64 at most, with
-// which the candidates of a query (k times the stride on average, within a
-// factor 1 +- 1 / sqrt(k)) stay below kMnCap for all but one query in 10^6.
-int many_stride_log2(int k) { return k <= 8 ? 3 : (k <= 20 ? 2 : (k <= 64 ? 1 : 0)); }
-
 int64_t many_pitch(const vie_head *hd, int k) {
-    const int64_t st = 8 << many_stride_log2(k);
+    const int64_t st = 8 << vie::many_stride_log2(k);
     return ((hd->V + st - 1) / st + 31) / 32 * 32;
 }
 
@@ -714,7 +709,7 @@ static vie_status run_topk_tc(const char *fn, vie_head *head, const float *h, in
 // Many queries: blocks of the filtered GEMM (vie_tc_many.cuh).
 static vie_status run_topk_many(const char *fn, vie_head *head, const float *h, int32_t batch, int32_t k,
                                 int32_t *out_idx, float *out_logits, float *sparse, cudaStream_t s) {
-    const int si = many_stride_log2(k), stride = 8 << si, block = many_block(head, k);
+    const int si = vie::many_stride_log2(k), stride = 8 << si, block = many_block(head, k);
     const int rows = static_cast<int>((head->V + stride - 1) / stride);
     const int64_t pitch = many_pitch(head, k);
     float *sample = reinterpret_cast<float *>(head->cand);  // read for the bounds before candidates replace it

@@ -25,4 +25,22 @@ constexpr int tc_bound_blocks(int slots, int k, int G) {
 }
 static_assert(bound_words_fit(64, 4) && bound_words_fit(8, 8), "the widest tensor-core and streaming launches");
 
+// ---- many queries: the sample ----
+constexpr int kMnCap = 2048;   // candidates kept per query
+constexpr int kMnMaxK = 128;
+
+// The sample takes every (8 << i)-th row, 64 at most.  A query's bound is its
+// r-th largest sampled logit, r >= k, and its candidates are the keys at or above
+// that: r times the stride on average, and more than kMnCap where fewer than r of
+// the kMnCap best keys were sampled, a binomial tail.  The largest r per stride
+// for which that happens to at most one query in 10^6:
+constexpr int kMnMaxRank[4] = {188, 79, 30, 9};
+constexpr int many_stride_log2(int k) { return k <= 8 ? 3 : (k <= 20 ? 2 : (k <= 64 ? 1 : 0)); }
+// The largest rank the bounds kernel accepts: its histogram finds the bin of the
+// k-th largest, and the smallest logit of that bin serves when few keys share it.
+constexpr int many_max_rank(int k) {
+    const int slack = k + k / 4 + 4, most = kMnMaxRank[many_stride_log2(k)];
+    return slack < most ? slack : most;
+}
+
 }  // namespace vie

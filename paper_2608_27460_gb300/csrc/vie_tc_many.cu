@@ -237,15 +237,16 @@ struct SampleKeys {
 // that none of their logits pass), count[q] = 0.  The sampled logits are read
 // once, into registers; a histogram over the upper half of their range gives
 // the bin of the k-th largest, and the smallest logit of that bin and those
-// above it is the bound.  Where that bin holds many keys (ties, outliers), or
-// the sample more than the registers, a radix select finds the exact k-th key
-// (13.3 us per 512 queries of 2374 sampled rows).
+// above it is the bound.  Where that would be a bound of more than max_rank
+// sampled keys (ties, outliers; many_max_rank), or the sample has more rows than
+// the registers hold, a radix select finds the exact k-th key (13.3 us per 512
+// queries of 2374 sampled rows).
 constexpr int kTauThreads = 512;
 template <int PER>
 __global__ void __launch_bounds__(kTauThreads, PER <= 8 ? 3 : 1) many_tau_kernel(const float *__restrict__ sample, int64_t pitch, int rows,
-                                                               uint32_t stride, int nq, int k, uint64_t *tau, float *tau_v,
-                                                               uint32_t *count) {
-    constexpr int kBins = 1024, kSlack = 4;
+                                                               uint32_t stride, int nq, int k, int max_rank, uint64_t *tau,
+                                                               float *tau_v, uint32_t *count) {
+    constexpr int kBins = 1024;
     __shared__ uint32_t hist[kBins];
     __shared__ uint32_t range[4];  // lowest, highest ordered logit, the k-th largest's bin (+ 1; 0: crowded), bound
     __shared__ MiscSmem ms;
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(kTauThreads, PER <= 8 ? 3 : 1) many_tau_kernel
                 if (run < uk && uk <= incl) {
                     int b = b0 + 31;
                     while (run + hist[b] < uk) run += hist[b--];
-                    if (run + hist[b] <= uk + uk / kSlack + kSlack) range[2] = static_cast<uint32_t>(b) + 1u;
+                    if (run + hist[b] <= static_cast<uint32_t>(max_rank)) range[2] = static_cast<uint32_t>(b) + 1u;
                 }
             }
             __syncthreads();
@@ -435,7 +436,7 @@ cudaError_t launch_many_tau(const float *sample, int64_t pitch, int rows, int st
                             uint64_t *tau, float *tau_v, uint32_t *count, cudaStream_t stream) {
     const auto kern = rows <= 8 * kTauThreads ? many_tau_kernel<8> : many_tau_kernel<32>;
     return launch_pdl(kern, dim3(static_cast<unsigned>(slots)), dim3(kTauThreads), 0, stream, sample, pitch, rows,
-                      static_cast<uint32_t>(stride), nq, k, tau, tau_v, count);
+                      static_cast<uint32_t>(stride), nq, k, many_max_rank(k), tau, tau_v, count);
 }
 
 cudaError_t launch_many_final(const uint64_t *cand, const uint32_t *count, int nq, int k,

@@ -34,6 +34,7 @@
 #include <cuda.h>
 #include <cstdint>
 
+#include "vie_plan.h"
 
 namespace vie {
 
@@ -42,8 +43,6 @@ constexpr int kMnBlock = 512;      // queries of a block of launches, at most
 constexpr int kMnRows = 256;       // rows of a tile (a CTA pair)
 constexpr int kMnStages = 6;
 constexpr int kMnStageBytes = 2 * 128 * 128;  // per CTA: 128 rows of W and of the query matrix
-constexpr int kMnCap = 2048;       // candidates kept per query
-constexpr int kMnMaxK = 128;
 constexpr int kMnEpiWarps = 8;
 constexpr int kMnThreads = 32 * (2 + kMnEpiWarps);
 constexpr uint32_t kMnSmem = 1024 + kMnStages * kMnStageBytes + 1024;  // barriers, ring, its alignment

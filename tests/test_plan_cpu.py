@@ -38,3 +38,19 @@ def test_shared_bound_words_stay_within_their_room(tmp_path):
                 if (b == 0 && G >= k) std::printf("unused %d %d %d\\n", slots, k, G);
             }""")
     assert not out, out[:10]
+
+
+def test_candidates_of_many_queries_seldom_overflow(tmp_path):
+    """The bound of a query is its r-th largest sampled logit, r at most the rank
+    the bounds kernel accepts.  More than `cap` keys reach it exactly when fewer
+    than r of the cap best keys were sampled, each with probability 1 / stride:
+    at most one query in 10^6, for every k."""
+    binom = pytest.importorskip("scipy.stats").binom
+    out = run_cpp(tmp_path, """
+    for (int k = 1; k <= kMnMaxK; ++k)
+        std::printf("%d %d %d %d\\n", k, 8 << many_stride_log2(k), many_max_rank(k), kMnCap);""")
+    assert len(out) == 128
+    for line in out:
+        k, stride, rank, cap = map(int, line.split())
+        assert rank >= k, line
+        assert binom.cdf(rank - 1, cap, 1.0 / stride) <= 1e-6, line
