@@ -465,7 +465,7 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
     const size_t cbytes =
         static_cast<size_t>(kMaxNB) * hd->G * (VIE_K_MAX + vie::kWideE) * sizeof(uint64_t);
     const size_t gbytes = static_cast<size_t>(hd->G) * vie::kBoundWords * sizeof(uint64_t);
-    const size_t mbytes = static_cast<size_t>(vie::kMnBlock) * (sizeof(uint64_t) + 2 * sizeof(float));
+    const size_t mbytes = static_cast<size_t>(vie::kMnBlock) * (sizeof(uint64_t) + 3 * sizeof(uint32_t));
     hd->cand_bytes = cbytes;
     hd->scratch_bytes = static_cast<int64_t>(cbytes + gbytes + mbytes + kNumWords * sizeof(uint32_t));
     e = cudaMalloc(&hd->W, wbytes);
@@ -716,6 +716,7 @@ static vie_status run_topk_many(const char *fn, vie_head *head, const float *h, 
     uint64_t *tau = head->gmax + static_cast<size_t>(head->G) * vie::kBoundWords;
     float *tau_v = reinterpret_cast<float *>(tau + vie::kMnBlock);
     uint32_t *count = reinterpret_cast<uint32_t *>(tau_v + vie::kMnBlock);
+    uint32_t *ticket = count + vie::kMnBlock;
     for (int q0 = 0; q0 < batch; q0 += block) {
         const int nq = batch - q0 < block ? batch - q0 : block;
         const int groups = (nq + vie::kMnGroup - 1) / vie::kMnGroup;
@@ -734,14 +735,16 @@ static vie_status run_topk_many(const char *fn, vie_head *head, const float *h, 
         p.sample_pitch = pitch;
         if (e == cudaSuccess) e = vie::launch_tc_many(head->mapS[si], head->mapHM, p, head->num_sms, s);
         if (e == cudaSuccess)
-            e = vie::launch_many_tau(sample, pitch, rows, stride, nq, groups * vie::kMnGroup, k, tau, tau_v, count, s);
+            e = vie::launch_many_tau(sample, pitch, rows, stride, nq, groups * vie::kMnGroup, k, tau, tau_v, count,
+                                     ticket, s);
         p.rows = head->V;
         p.sample = nullptr;
         if (e == cudaSuccess) e = vie::launch_tc_many(head->mapW, head->mapHM, p, head->num_sms, s);
+        const int64_t o = static_cast<int64_t>(q0) * k;
         if (e == cudaSuccess)
-            e = vie::launch_many_final(head->cand, count, nq, k, head->W, head->V, head->d, head->d_pad, hq,
-                                       out_idx + static_cast<int64_t>(q0) * k, out_logits + static_cast<int64_t>(q0) * k,
-                                       sparse != nullptr ? sparse + static_cast<int64_t>(q0) * head->V : nullptr, s);
+            e = vie::launch_many_final({head->cand, count, ticket, nq, k, head->W, head->V, head->d, head->d_pad, hq,
+                                        out_idx + o, out_logits + o,
+                                        sparse != nullptr ? sparse + static_cast<int64_t>(q0) * head->V : nullptr}, s);
         if (e != cudaSuccess) return fail_cuda(e, fn);
     }
     return VIE_OK;

@@ -37,6 +37,7 @@ cudaError_t launch_stream_topk_e4m3_nb8(int r, const StreamTopkParams &p, int gr
 // ---- tensor-core head (vie_tc_topk.cu, vie_tc_many.cu) ----
 struct TcParams;
 struct MnParams;
+struct MnFinalParams;
 
 // The filtered GEMM for many queries: one launch of the GEMM (sample or main),
 // the bounds from the sample's logits (slots = 128 per query group), and the
@@ -44,10 +45,8 @@ struct MnParams;
 cudaError_t launch_tc_many(const CUtensorMap &mapW, const CUtensorMap &mapH, const MnParams &p, int sms,
                            cudaStream_t stream);
 cudaError_t launch_many_tau(const float *sample, int64_t pitch, int rows, int stride, int nq, int slots, int k,
-                            uint64_t *tau, float *tau_v, uint32_t *count, cudaStream_t stream);
-cudaError_t launch_many_final(const uint64_t *cand, const uint32_t *count, int nq, int k,
-                              const void *W, int64_t V, int d, int d_pad, const float *h, int32_t *out_idx,
-                              float *out_logits, float *sparse, cudaStream_t stream);
+                            uint64_t *tau, float *tau_v, uint32_t *count, uint32_t *ticket, cudaStream_t stream);
+cudaError_t launch_many_final(const MnFinalParams &p, cudaStream_t stream);
 
 // Recall@k: per query, how many exact top-k indices the candidates contain.
 cudaError_t launch_recall_hits(const int32_t *exact, int k, const int32_t *approx, int m, int64_t n,

@@ -234,7 +234,7 @@ struct SampleKeys {
 
 // One CTA per query slot of the block: tau[q] = a key with at least k sampled
 // keys at or above it, tau_v[q] its logit (+inf for slots without a query, so
-// that none of their logits pass), count[q] = 0.  The sampled logits are read
+// that none of their logits pass), count[q] = ticket[q] = 0.  The sampled logits are read
 // once, into registers; a histogram over the upper half of their range gives
 // the bin of the k-th largest, and the smallest logit of that bin and those
 // above it is the bound.  Where that would be a bound of more than max_rank
@@ -245,7 +245,7 @@ constexpr int kTauThreads = 512;
 template <int PER>
 __global__ void __launch_bounds__(kTauThreads, PER <= 8 ? 3 : 1) many_tau_kernel(const float *__restrict__ sample, int64_t pitch, int rows,
                                                                uint32_t stride, int nq, int k, int max_rank, uint64_t *tau,
-                                                               float *tau_v, uint32_t *count) {
+                                                               float *tau_v, uint32_t *count, uint32_t *ticket) {
     constexpr int kBins = 1024;
     __shared__ uint32_t hist[kBins];
     __shared__ uint32_t range[4];  // lowest, highest ordered logit, the k-th largest's bin (+ 1; 0: crowded), bound
@@ -332,83 +332,190 @@ __global__ void __launch_bounds__(kTauThreads, PER <= 8 ? 3 : 1) many_tau_kernel
         // (below order_f32(-FLT_MAX) there are only -inf and NaN patterns)
         tau_v[q] = q >= nq ? __uint_as_float(0x7F800000u) : (hi < 0x00800000u ? __uint_as_float(0xFF800000u) : unorder_f32(hi));
         count[q] = 0;
+        ticket[q] = 0;
     }
 }
 
-// One CTA per query: the exact top-k of its candidates, best first, and its
-// row of the sparse tensor.  A list that overflowed is replaced by the best of
-// all rows, computed here (fp32 dot products, one warp per row).
-__global__ void __launch_bounds__(kThreads) many_final_kernel(const uint64_t *cand, const uint32_t *count,
-                                                             int k, const uint16_t *W,
-                                                             int64_t V, int d, int d_pad, const float *h,
-                                                             int32_t *out_idx, float *out_logits, float *sparse) {
-    extern __shared__ __align__(16) unsigned char fin_smem[];
-    __shared__ MiscSmem ms;
+// The best k of the logits of rows [r0, r1) of W against hq, and often a few
+// more, to mb.cands; returns how many there are.  fp32 dot products, four rows per warp at a
+// time, 16 bytes per lane and row: 20 KB in flight per CTA, four CTAs per SM.
+static __device__ __forceinline__ int rescan_rows(const uint16_t *W, int64_t r0, int64_t r1, int d, int d_pad,
+                                               const float *hq, int k, const MergeBufs &mb, MiscSmem *ms) {
+    constexpr int kWarps = kThreads / 32, kRows = 4;
+    constexpr int kRound = kMergeCandCap / 2;  // rows between cut-backs; k <= kMnMaxK keys stay
+    static_assert(kMnMaxK <= kRound, "a round's keys and those kept fit the buffer");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int C = d_pad >> 3;
+    const bool vec = (reinterpret_cast<uintptr_t>(hq) & 15u) == 0;
+    uint64_t bound = 1;
+    if (tid == 0) ms->n_cand = 0;
+    __syncthreads();
+    int n = 0;
+    for (int64_t a = r0; a < r1; a += kRound) {
+        const int rows = static_cast<int>(min(static_cast<int64_t>(kRound), r1 - a));
+        const uint4 *Wa = reinterpret_cast<const uint4 *>(W) + a * C;
+        for (int b = kRows * warp; b < rows; b += kRows * kWarps) {
+            float acc[kRows] = {};
+#pragma unroll 1
+            for (int c = lane; c < C; c += 32) {
+                uint4 w[kRows];
+#pragma unroll
+                for (int i = 0; i < kRows; ++i)
+                    w[i] = __ldg(Wa + static_cast<int64_t>(min(b + i, rows - 1)) * C + c);
+                float x[8];
+                if (vec && 8 * c + 8 <= d) {
+                    const float4 lo = __ldg(reinterpret_cast<const float4 *>(hq) + 2 * c);
+                    const float4 hi = __ldg(reinterpret_cast<const float4 *>(hq) + 2 * c + 1);
+                    x[0] = lo.x, x[1] = lo.y, x[2] = lo.z, x[3] = lo.w;
+                    x[4] = hi.x, x[5] = hi.y, x[6] = hi.z, x[7] = hi.w;
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) x[e] = 8 * c + e < d ? __ldg(hq + 8 * c + e) : 0.0f;
+                }
+#pragma unroll
+                for (int i = 0; i < kRows; ++i) {
+                    acc[i] = fmaf(bf16_lo(w[i].x), x[0], acc[i]);
+                    acc[i] = fmaf(bf16_hi(w[i].x), x[1], acc[i]);
+                    acc[i] = fmaf(bf16_lo(w[i].y), x[2], acc[i]);
+                    acc[i] = fmaf(bf16_hi(w[i].y), x[3], acc[i]);
+                    acc[i] = fmaf(bf16_lo(w[i].z), x[4], acc[i]);
+                    acc[i] = fmaf(bf16_hi(w[i].z), x[5], acc[i]);
+                    acc[i] = fmaf(bf16_lo(w[i].w), x[6], acc[i]);
+                    acc[i] = fmaf(bf16_hi(w[i].w), x[7], acc[i]);
+                }
+            }
+            uint64_t key = 0;
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                float z = acc[i];
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+                if (lane == i && b + i < rows) key = make_key(z, static_cast<uint32_t>(a) + static_cast<uint32_t>(b + i));
+            }
+            if (key >= bound) mb.cands[atomicAdd(&ms->n_cand, 1)] = key;
+        }
+        __syncthreads();
+        n = ms->n_cand;
+        __syncthreads();  // read by all before the next round adds to it
+        if (n > k && (n > kRound || a + kRound >= r1)) {  // keep the best k
+            const uint64_t T = block_radix_threshold(SmemKeys{mb.cands}, n, k, 1, mb.hist, ms);
+            if (tid == 0) ms->n_win = 0;
+            __syncthreads();
+            for (int i = tid; i < n; i += kThreads)
+                if (mb.cands[i] >= T) mb.win[atomicAdd(&ms->n_win, 1)] = mb.cands[i];
+            __syncthreads();
+            for (int i = tid; i < k; i += kThreads) mb.cands[i] = mb.win[i];
+            bound = T;
+            n = k;
+            if (tid == 0) ms->n_cand = k;
+            __syncthreads();
+        }
+    }
+    return n;
+}
+
+// The buffers of a merge in mem (SmemLayout::merge_fixed_bytes()).
+static __device__ __forceinline__ MergeBufs merge_bufs(unsigned char *mem) {
     MergeBufs mb;
-    mb.pref = reinterpret_cast<uint64_t *>(fin_smem);
+    mb.pref = reinterpret_cast<uint64_t *>(mem);
     mb.cands = mb.pref + kMergePrefixCap;
     mb.win = mb.cands + kMergeCandCap;
     mb.counts = reinterpret_cast<int *>(mb.win + 1024);
     mb.offsets = mb.counts + kMaxLists;
     mb.hist = reinterpret_cast<uint32_t *>(mb.offsets + kMaxLists);
-    griddep_launch_dependents();
-    griddep_wait();
-    const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float *sp = nullptr;
-    if (sparse != nullptr) {
-        sp = sparse + q * V;
-        for (int64_t i = tid; i < V; i += kThreads) sp[i] = __uint_as_float(0xFF800000u);
-    }
-    const uint64_t *list = cand + static_cast<size_t>(q) * kMnCap;
-    const uint32_t n_all = count[q];
-    if (tid == 0) {
-        ms.n_win = 0;
-        ms.n_cand = 0;
+    return mb;
+}
+
+// Whether a query's list of n candidates holds its top k (too many were not
+// kept; too few are logits that are not numbers).
+static __device__ __forceinline__ bool complete(uint32_t n, int k) {
+    return n >= static_cast<uint32_t>(k) && n <= kMnCap;
+}
+
+// Query q's row of the sparse tensor, -inf so far; nullptr without one.
+static __device__ __forceinline__ float *fill_sparse(const MnFinalParams &p, int q) {
+    if (p.sparse == nullptr) return nullptr;
+    float *sp = p.sparse + q * p.V;
+    for (int64_t i = threadIdx.x; i < p.V; i += kThreads) sp[i] = __uint_as_float(0xFF800000u);
+    return sp;
+}
+
+// The queries without a complete list, recomputed from all rows.  All CTAs of
+// the launch share the work: kMnCap / k slices of the rows per such query, the
+// k best of each slice to the query's own list, and the CTA that finishes the
+// last slice ranks them (a ticket; nobody waits).
+static __device__ __noinline__ void rescan_queries(const MnFinalParams &p, unsigned char *mem, MiscSmem *ms) {
+    __shared__ uint16_t missed[kMnBlock];
+    __shared__ int n_missed, last;
+    const MergeBufs mb = merge_bufs(mem);
+    const int tid = threadIdx.x, lane = tid & 31, k = p.k;
+    if (tid < 32) {  // in the same order in every CTA
+        int n = 0;
+        for (int i0 = 0; i0 < p.nq; i0 += 32) {
+            const bool m = i0 + lane < p.nq && !complete(p.count[i0 + lane], k);
+            const unsigned mask = __ballot_sync(0xFFFFFFFFu, m);
+            if (m) missed[n + __popc(mask & ((1u << lane) - 1u))] = static_cast<uint16_t>(i0 + lane);
+            n += __popc(mask);
+        }
+        if (lane == 0) n_missed = n;
     }
     __syncthreads();
-    static_assert(kMnCap <= kMergeCandCap, "a query's candidates are ranked in shared memory");
-    int n;
-    if (n_all >= static_cast<uint32_t>(k) && n_all <= kMnCap) {
-        n = static_cast<int>(n_all);
-        for (int i = tid; i < n; i += kThreads) mb.cands[i] = __ldcg(reinterpret_cast<const unsigned long long *>(list) + i);
-    } else {
-        const float *hq = h + static_cast<int64_t>(q) * d;
-        constexpr int kRound = kMergeCandCap / 2;  // rows between cut-backs; k <= 1024 stay
-        uint64_t bound = 1;  // (tau is a tensor-core logit: these sums may fall a rounding short of it)
-        for (int64_t r0 = 0; r0 < V; r0 += kRound) {
-            const int64_t r1 = min(V, r0 + kRound);
-            for (int64_t r = r0 + warp; r < r1; r += kThreads / 32) {
-                const uint16_t *wr = W + r * d_pad;
-                float a = 0.0f;
-                for (int j = lane; j < d; j += 32) a = fmaf(__uint_as_float(static_cast<uint32_t>(wr[j]) << 16), hq[j], a);
-#pragma unroll
-                for (int o = 16; o >= 1; o >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-                const uint64_t key = make_key(a, static_cast<uint32_t>(r));
-                if (lane == 0 && key >= bound) mb.cands[atomicAdd(&ms.n_cand, 1)] = key;
+    const int slices = min(kMnCap / k, 256), tasks = slices * n_missed;
+    const int64_t share = (p.V + slices - 1) / slices;
+    for (int t = blockIdx.x; t < tasks; t += gridDim.x) {
+        const int s = t / n_missed, q = missed[t - s * n_missed];
+        const int64_t r0 = min(p.V, s * share), r1 = min(p.V, r0 + share);
+        const int n = rescan_rows(p.W, r0, r1, p.d, p.d_pad, p.h + static_cast<int64_t>(q) * p.d, k, mb, ms);
+        uint64_t *list = p.cand + static_cast<size_t>(q) * kMnCap;
+        for (int i = tid; i < k; i += kThreads) list[s * k + i] = i < n ? mb.cands[i] : 0ull;
+        __syncthreads();  // orders the slice's keys before thread 0's ticket
+        if (tid == 0) {
+            last = atomic_add_acq_rel_gpu(p.ticket + q, 1u) == static_cast<uint32_t>(slices - 1) ? 1 : 0;
+            ms->n_cand = 0;
+        }
+        __syncthreads();
+        if (last) {
+            float *sp = fill_sparse(p, q);
+            for (int i = tid; i < slices * k; i += kThreads) {
+                const uint64_t x = __ldcg(reinterpret_cast<const unsigned long long *>(list) + i);
+                if (x != 0) mb.cands[atomicAdd(&ms->n_cand, 1)] = x;
             }
             __syncthreads();
-            const int m = ms.n_cand;
-            __syncthreads();  // read by all before the next round adds to it
-            if (m > kMergeCandCap / 2) {  // keep the best k
-                const uint64_t T = block_radix_threshold(SmemKeys{mb.cands}, m, k, 1, mb.hist, &ms);
-                for (int i = tid; i < m; i += kThreads)
-                    if (mb.cands[i] >= T) mb.win[atomicAdd(&ms.n_win, 1)] = mb.cands[i];
-                __syncthreads();
-                for (int i = tid; i < k; i += kThreads) mb.cands[i] = mb.win[i];
-                bound = T;
-                __syncthreads();
-                if (tid == 0) {
-                    ms.n_win = 0;
-                    ms.n_cand = k;
-                }
-                __syncthreads();
-            }
+            block_topk_to_output(mb.cands, ms->n_cand, k, mb, ms, p.out_idx + static_cast<int64_t>(q) * k,
+                                 p.out_logits + static_cast<int64_t>(q) * k, sp);
         }
-        n = ms.n_cand;
+        __syncthreads();  // the buffers are free for the next task
     }
-    __syncthreads();
-    block_topk_to_output(mb.cands, n, k, mb, &ms, out_idx + static_cast<int64_t>(q) * k,
-                         out_logits + static_cast<int64_t>(q) * k, sp);
+}
+
+// One CTA per query: the exact top-k of its candidates, best first, and its
+// row of the sparse tensor; then the queries whose lists overflowed, together.
+// One such query of 512 adds 0.23 ms at 151936 x 1024, k = 2 (33 ms when its own
+// CTA recomputed it alone, two bytes at a time) and 2.7 ms at 128256 x 3072, k =
+// 50, 40 slices (80 ms); all 512 of them take 28 and 124 ms (43 and 234 ms).
+// (Four CTAs per SM: with the registers that the recomputation would like, two
+// would fit, and every block pays for that.)
+__global__ void __launch_bounds__(kThreads, 4) many_final_kernel(const __grid_constant__ MnFinalParams p) {
+    extern __shared__ __align__(16) unsigned char fin_smem[];
+    __shared__ MiscSmem ms;
+    griddep_launch_dependents();
+    griddep_wait();
+    const int q = blockIdx.x, tid = threadIdx.x, k = p.k;
+    const uint32_t n = p.count[q];
+    bool miss = false;
+    for (int i = tid; i < p.nq; i += kThreads) miss |= !complete(p.count[i], k);
+    static_assert(kMnCap <= kMergeCandCap, "a query's candidates are ranked in shared memory");
+    if (complete(n, k)) {
+        float *sp = fill_sparse(p, q);
+        const MergeBufs mb = merge_bufs(fin_smem);
+        const uint64_t *list = p.cand + static_cast<size_t>(q) * kMnCap;
+        for (int i = tid; i < static_cast<int>(n); i += kThreads)
+            mb.cands[i] = __ldcg(reinterpret_cast<const unsigned long long *>(list) + i);
+        __syncthreads();
+        block_topk_to_output(mb.cands, static_cast<int>(n), k, mb, &ms, p.out_idx + static_cast<int64_t>(q) * k,
+                             p.out_logits + static_cast<int64_t>(q) * k, sp);
+    }
+    if (__syncthreads_or(miss ? 1 : 0)) rescan_queries(p, fin_smem, &ms);
 }
 
 cudaError_t launch_tc_many(const CUtensorMap &mapW, const CUtensorMap &mapH, const MnParams &p, int sms,
@@ -433,18 +540,15 @@ cudaError_t launch_tc_many(const CUtensorMap &mapW, const CUtensorMap &mapH, con
 }
 
 cudaError_t launch_many_tau(const float *sample, int64_t pitch, int rows, int stride, int nq, int slots, int k,
-                            uint64_t *tau, float *tau_v, uint32_t *count, cudaStream_t stream) {
+                            uint64_t *tau, float *tau_v, uint32_t *count, uint32_t *ticket, cudaStream_t stream) {
     const auto kern = rows <= 8 * kTauThreads ? many_tau_kernel<8> : many_tau_kernel<32>;
     return launch_pdl(kern, dim3(static_cast<unsigned>(slots)), dim3(kTauThreads), 0, stream, sample, pitch, rows,
-                      static_cast<uint32_t>(stride), nq, k, many_max_rank(k), tau, tau_v, count);
+                      static_cast<uint32_t>(stride), nq, k, many_max_rank(k), tau, tau_v, count, ticket);
 }
 
-cudaError_t launch_many_final(const uint64_t *cand, const uint32_t *count, int nq, int k,
-                              const void *W, int64_t V, int d, int d_pad, const float *h, int32_t *out_idx,
-                              float *out_logits, float *sparse, cudaStream_t stream) {
-    return launch_pdl(many_final_kernel, dim3(static_cast<unsigned>(nq)), dim3(kThreads),
-                      SmemLayout::merge_fixed_bytes(), stream, cand, count, k,
-                      static_cast<const uint16_t *>(W), V, d, d_pad, h, out_idx, out_logits, sparse);
+cudaError_t launch_many_final(const MnFinalParams &p, cudaStream_t stream) {
+    return launch_pdl(many_final_kernel, dim3(static_cast<unsigned>(p.nq)), dim3(kThreads),
+                      SmemLayout::merge_fixed_bytes(), stream, p);
 }
 
 }  // namespace vie

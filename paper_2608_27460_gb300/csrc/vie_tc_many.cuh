@@ -13,8 +13,8 @@
 //   final   per query, the exact top-k of its candidates.
 // The sample takes every s-th row of the total order's index range, and tau is
 // a key (logit, then row), so neither ties nor clusters of neighbouring rows
-// make many candidates; a list that overflows all the same (kMnCap) is
-// recomputed row by row by its query's CTA.  20000 queries, 151936 x 1024,
+// make many candidates; a query whose list overflows all the same (kMnCap)
+// is recomputed from all rows by the CTAs of the final launch.  20000 queries, 151936 x 1024,
 // k = 2: 22.0 ms in passes of 64 queries, 9.1 ms here (per 512 queries: main
 // 194 us, 1.64 PFLOP/s; the other four launches ~30 us).
 //
@@ -58,6 +58,20 @@ struct MnParams {
     uint64_t *cand;        // [query][kMnCap] keys
     uint32_t *count;       // [query]
     uint32_t *err;
+};
+
+struct MnFinalParams {
+    uint64_t *cand;         // [query][kMnCap] keys
+    const uint32_t *count;  // [query] candidates that reached the bound
+    uint32_t *ticket;       // [query] slices finished, 0 before the launch
+    int32_t nq, k;
+    const uint16_t *W;      // [V][d_pad] bf16 bits
+    int64_t V;
+    int32_t d, d_pad;
+    const float *h;         // [nq][d]
+    int32_t *out_idx;       // [nq][k]
+    float *out_logits;      // [nq][k]
+    float *sparse;          // [nq][V] or nullptr
 };
 
 }  // namespace vie

@@ -135,6 +135,70 @@ def test_many_queries_whose_candidates_overflow(vie, k):
     np.testing.assert_array_equal(idx[3], np.arange(k))
 
 
+def _rare_low_rows(V, d, n, low, seed):
+    """Every 8th row (all that a sample of any stride takes) has -1 in column 0
+    and the others +1; the queries in `low` are mostly that column, so seven
+    eighths of the rows reach their sampled bound."""
+    W, h = workload(V, d, n, seed=seed)
+    f = synth.bf16_bits_to_f32(W)
+    f[:, 0] = 1.0
+    f[::8, 0] = -1.0
+    h[:, 0] = 0.0
+    h[low] *= 0.01
+    h[low, 0] = 5.0
+    return synth.f32_to_bf16_bits(f), h
+
+
+@pytest.mark.parametrize("V,d,batch,low,k", [
+    (8192, 64, 256, [7], 1),               # 256 slices of 32 rows
+    (20011, 100, 257, [0, 255, 256], 50),  # 40 slices; rows that are no multiple of 16 bytes of h
+    (30000, 72, 513, [512], 8),            # alone in the second block of launches
+    (20011, 264, 300, list(range(0, 300, 2)), 128),  # 16 slices of more rows than one round
+])
+def test_many_queries_some_recomputed(vie, V, d, batch, low, k):
+    """Queries whose candidates overflow are recomputed by all CTAs of the
+    final launch, among queries that are not; the sparse rows of both."""
+    import torch
+    W, h = _rare_low_rows(V, d, batch, low, seed=V + k)
+    z = oracle.logits(W, h)
+    with vie.Head(to_device_bits(W)) as head:
+        hd = torch.from_numpy(h).cuda()
+        for _ in range(2):  # the counters are re-armed
+            i, v, sp = head.topk_sparse(hd, k)
+            want = head.sparse_logits(i, v)
+            torch.cuda.synchronize()
+            assert head.device_status() == vie.VIE_OK
+            np.testing.assert_array_equal(sp.cpu().numpy().view(np.uint32), want.cpu().numpy().view(np.uint32))
+            idx, val = i.cpu().numpy(), v.cpu().numpy()
+            for q in range(batch):
+                assert not check_topk(idx[q], val[q], z[q], k), q
+
+
+def test_a_recomputed_query_is_no_cliff(vie):
+    """One query of 512 whose candidates overflow: its rows are shared by the
+    CTAs of the launch (its own CTA alone took over 100 times the call)."""
+    import torch
+    V, d, batch, k = 100003, 512, 512, 2
+    W, h = _rare_low_rows(V, d, batch, [7], seed=9)
+    plain = h.copy()
+    plain[7] = plain[8]
+    with vie.Head(to_device_bits(W)) as head:
+        t = []
+        for x in (plain, h):
+            xd = torch.from_numpy(x).cuda()
+            out = head.topk(xd, k)
+            ms = []
+            for _ in range(5):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                head.topk(xd, k, out_idx=out[0], out_logits=out[1])
+                b.record()
+                b.synchronize()
+                ms.append(a.elapsed_time(b))
+            t.append(min(ms))
+    assert t[1] < 10 * t[0], t
+
+
 def test_many_queries_sparse_and_captured(vie):
     """The sparse rows of a filtered-GEMM call equal the scatter of its own
     top-k, and replaying the captured call gives the eager bits."""
