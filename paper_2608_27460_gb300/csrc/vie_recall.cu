@@ -13,7 +13,12 @@
 //   k <= 8   every lane keeps all k exact entries in registers and compares
 //            its own candidates with them (a bit per entry, OR-ed over the
 //            warp at the end);
-//   k > 8    the exact entries go into a hash table in shared memory (open
+//   k > 8 and m <= 32
+//            the other way round: every lane keeps all m candidates and
+//            compares its own exact entries with them (a table would be built
+//            for a few look-ups: n = 20000, k = 1000: 15 us at m = 1 instead
+//            of 90, 43 at m = 32 instead of 95);
+//   else     the exact entries go into a hash table in shared memory (open
 //            addressing, at most a quarter full), each with the number of
 //            positions that hold it; a candidate that finds its entry takes
 //            that number and leaves 0, so a repeat adds nothing.  Most
@@ -63,6 +68,36 @@ __global__ void __launch_bounds__(kRecallWarps * 32) recall_direct_kernel(const 
         if (e[j] < 0) found &= ~(1u << j);
     found = __reduce_or_sync(0xFFFFFFFFu, found);
     if (lane == 0) hits[q] = __popc(found);
+}
+
+// m <= M: one warp per query, exact entries lane, lane + 32, ..., U at a time.
+template <int M, int U>
+__global__ void __launch_bounds__(kRecallWarps * 32) recall_few_kernel(const int32_t *__restrict__ exact, int k,
+                                                                      const int32_t *__restrict__ approx, int m,
+                                                                      int64_t n, int32_t *__restrict__ hits) {
+    griddep_wait();  // the lists may come from the kernels before this one
+    const int lane = threadIdx.x & 31;
+    const int64_t q = static_cast<int64_t>(blockIdx.x) * kRecallWarps + (threadIdx.x >> 5);
+    if (q >= n) return;
+    const int32_t *eq = exact + q * k;
+    int32_t a[M];
+#pragma unroll
+    for (int j = 0; j < M; ++j) a[j] = j < m ? approx[q * m + j] : -1;
+    unsigned sum = 0;
+    for (int i0 = lane; i0 < k; i0 += 32 * U) {
+        int32_t e[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) e[u] = i0 + 32 * u < k ? eq[i0 + 32 * u] : -1;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            bool in = false;
+#pragma unroll
+            for (int j = 0; j < M; ++j) in |= e[u] == a[j];
+            sum += in && e[u] >= 0 ? 1u : 0u;  // an empty exact entry is never a hit
+        }
+    }
+    sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+    if (lane == 0) hits[q] = static_cast<int32_t>(sum);
 }
 
 // k > 8: WPQ warps per query (1, or all kRecallWarps of the CTA), a table of
@@ -169,6 +204,12 @@ cudaError_t launch_recall_hits(const int32_t *exact, int k, const int32_t *appro
     cfg.numAttrs = 1;
     if (k <= 2) return cudaLaunchKernelEx(&cfg, recall_direct_kernel<2>, exact, k, approx, m, n, hits);
     if (k <= 8) return cudaLaunchKernelEx(&cfg, recall_direct_kernel<8>, exact, k, approx, m, n, hits);
+    if (m <= 32) {
+        const auto few = m <= 8 ? (k <= 128 ? recall_few_kernel<8, 4> : recall_few_kernel<8, 8>)
+                                : (m <= 16 ? (k <= 128 ? recall_few_kernel<16, 4> : recall_few_kernel<16, 8>)
+                                           : (k <= 128 ? recall_few_kernel<32, 4> : recall_few_kernel<32, 8>));
+        return cudaLaunchKernelEx(&cfg, few, exact, k, approx, m, n, hits);
+    }
     int log2_slots = 6;
     while ((1 << log2_slots) < 4 * k) ++log2_slots;
     const size_t table = size_t(9) << log2_slots;

@@ -30,12 +30,14 @@ def _lists(n, k, m, seed, V=5000, share=0.5, empty=0.1, repeats=0.1, neg_exact=F
 
 @pytest.mark.parametrize("n,k,m", [
     (1, 1, 1), (37, 2, 2), (20000, 2, 2),     # Recall@2 over 20k states, as in Section 4.3
-    (257, 50, 64), (64, 33, 500),             # first k of 4 entries per lane
-    (20, 129, 1000),                          # first k of 32 entries per lane
+    (257, 50, 64), (64, 33, 500),             # a table per warp
+    (20, 129, 1000),                          # a table per CTA
+    (300, 9, 8), (300, 9, 9), (257, 1024, 1), # candidates in registers: 8, 16 or 32 of them
+    (4001, 129, 32), (300, 128, 16), (300, 128, 17), (300, 257, 16), (300, 129, 33),
     (5, 1024, 4096), (3, 1024, 1), (9, 32, 70000)])
 def test_hits_match_the_oracle(vie, n, k, m):
     import torch
-    ex, ap = _lists(n, k, m, seed=n * 7 + k * 3 + m, neg_exact=(k == 33))
+    ex, ap = _lists(n, k, m, seed=n * 7 + k * 3 + m, neg_exact=(k in (9, 33, 129)))
     got = vie.recall_hits(torch.from_numpy(ex).cuda(), torch.from_numpy(ap).cuda())
     torch.cuda.synchronize()
     np.testing.assert_array_equal(got.cpu().numpy(), oracle.recall_hits(ex, ap))
@@ -64,6 +66,31 @@ def test_hits_with_colliding_and_repeated_entries(vie, n, k, m):
     torch.cuda.synchronize()
     rows = np.arange(n) if n * k * m < 2e8 else np.arange(0, n, 5)
     np.testing.assert_array_equal(got.cpu().numpy()[rows], oracle.recall_hits(ex[rows], ap[rows]))
+
+
+def test_few_candidates_cost_no_more_than_reading_the_lists(vie):
+    """k = 1000 exact entries against one candidate: bound by the 80 MB of exact
+    lists (a copy of them, twice the bytes, is the yardstick)."""
+    import torch
+    ex = torch.randint(0, 150000, (20000, 1000), dtype=torch.int32, device="cuda")
+    ap = torch.randint(0, 150000, (20000, 1), dtype=torch.int32, device="cuda")
+    dst = torch.empty_like(ex)
+
+    def fastest(f):
+        f()
+        ms = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                f()
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        return min(ms)
+
+    t, copy = fastest(lambda: vie.recall_hits(ex, ap)), fastest(lambda: dst.copy_(ex))
+    assert t < 2 * copy, (t, copy)
 
 
 def test_hits_edge_lists(vie):
