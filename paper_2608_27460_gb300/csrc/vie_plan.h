@@ -17,11 +17,16 @@ constexpr int kBoundWords = 256;  // words per CTA: 64 slots x 4 on the tensor-c
 constexpr bool bound_words_fit(int slots, int blocks) { return slots * blocks <= kBoundWords; }
 
 // Maxima per CTA and query of a tensor-core launch of `slots` query slots on G
-// CTAs: one per tile, or four (of 32 rows each) where one from every CTA would
-// be too few for k; none (0) where neither gives k of them.
-constexpr int tc_bound_blocks(int slots, int k, int G) {
-    const int b = 2 * k <= G || !bound_words_fit(slots, 4) ? 1 : 4;
-    return b * G >= k && b * G <= kBoundMax && bound_words_fit(slots, b) ? b : 0;
+// CTAs and so many tiles of W: one of each CTA's first tile, or four (of 32
+// rows each) where one from every CTA with a tile would be fewer than 2 k; none
+// (0) where four give less than k and a quarter: the bound then lies so low, or
+// is never reached, that waiting for it costs more than it saves (V = 2000, 16
+// tiles, 64 maxima, b = 4: k = 50 39.8 us without and 17.3 with, k = 64 45.3
+// and 48.5, k = 65, where there are too few, 44.7 and 56.2).
+constexpr int tc_bound_blocks(int slots, int k, int G, int64_t tiles) {
+    const int n = tiles < G ? static_cast<int>(tiles) : G;  // CTAs that publish
+    const int b = 2 * k <= n || !bound_words_fit(slots, 4) ? 1 : 4;
+    return 4 * b * n >= 5 * k && b * G <= kBoundMax && bound_words_fit(slots, b) ? b : 0;
 }
 static_assert(bound_words_fit(64, 4) && bound_words_fit(8, 8), "the widest tensor-core and streaming launches");
 
