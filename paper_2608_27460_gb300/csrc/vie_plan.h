@@ -17,16 +17,16 @@ constexpr int kBoundWords = 256;  // words per CTA: 64 slots x 4 on the tensor-c
 constexpr bool bound_words_fit(int slots, int blocks) { return slots * blocks <= kBoundWords; }
 
 // Maxima per CTA and query of a tensor-core launch of `slots` query slots on G
-// CTAs and so many tiles of W: one of each CTA's first tile, or four (of 32
-// rows each) where one from every CTA with a tile would be fewer than 2 k; none
-// (0) where four give less than k and a quarter: the bound then lies so low, or
-// is never reached, that waiting for it costs more than it saves (V = 2000, 16
-// tiles, 64 maxima, b = 4: k = 50 39.8 us without and 17.3 with, k = 64 45.3
-// and 48.5, k = 65, where there are too few, 44.7 and 56.2).
-constexpr int tc_bound_blocks(int slots, int k, int G, int64_t tiles) {
-    const int n = tiles < G ? static_cast<int>(tiles) : G;  // CTAs that publish
-    const int b = 2 * k <= n || !bound_words_fit(slots, 4) ? 1 : 4;
-    return 4 * b * n >= 5 * k && b * G <= kBoundMax && bound_words_fit(slots, b) ? b : 0;
+// CTAs, V rows of W in tiles of 128: one of each CTA's first tile, or four (of
+// 32 rows each) where G is below 2 k (evaluating four times the words is slower
+// where one will do: 12000 rows, 64 queries, k = 50: 32.5 us with one, 54.5 with
+// four); none (0) where the rows do not give k of them, which every launch
+// would wait for in vain.
+constexpr int tc_bound_blocks(int slots, int k, int G, int64_t V) {
+    const int b = 2 * k <= G || !bound_words_fit(slots, 4) ? 1 : 4;
+    const int64_t blocks = b == 1 ? (V + 127) / 128 : (V + 31) / 32;  // words there can be
+    const int64_t words = blocks < b * G ? blocks : b * G;
+    return words >= k && b * G <= kBoundMax && bound_words_fit(slots, b) ? b : 0;
 }
 static_assert(bound_words_fit(64, 4) && bound_words_fit(8, 8), "the widest tensor-core and streaming launches");
 
