@@ -43,6 +43,8 @@ def test_plan_selects_paths(vie):
     (64, 128, 2, 64),        # k = V on one CTA
     (200, 256, 40, 64),      # 64-query tile over two tiles
     (129, 128, 8, 128),      # largest k, a one-row last tile
+    (2000, 256, 4, 128),     # every row is a candidate: logits of both signs crowd the ranking's bins
+    (600, 128, 4, 100),      # the same, few enough to rank by all pairs
 ])
 def test_tensor_core_parity(vie, V, d, batch, k):
     W, h = workload(V, d, batch, seed=V + batch + k)

@@ -28,6 +28,8 @@ def streaming(vie):
     (100003, 128, 5, 300, 2),   # groups of 4 + 1 (640-key buffers)
     (50021, 256, 2, 1024, 1),   # two 2048-key buffers, k = 1024
     (7001, 640, 1, 65, 1),      # fewer rows per CTA than the buffer holds
+    (1500, 64, 1, 700, 1),      # nearly every row a candidate, of both signs: a sort of the best k
+    (2000, 64, 3, 300, 1),      # the same, ranked by all pairs
 ])
 def test_wide_lists_match_the_oracle(vie, V, d, batch, k, launches):
     W, h = workload(V, d, batch, seed=V + k)
