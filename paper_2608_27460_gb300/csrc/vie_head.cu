@@ -691,7 +691,7 @@ static vie_status run_topk_tc(const char *fn, vie_head *head, const float *h, in
         p.flags = head->words + kFlagWords;
         p.counts = head->words + kCountWords;
         p.gmax = head->gmax;
-        p.gt_blocks = vie::tc_bound_blocks(nqt, k, head->G, head->V);
+        p.gt_blocks = vie::tc_bound_blocks(nqt, k, head->G, head->V, head->d_pad * (q8 ? 1 : 2));
         p.out_idx = out_idx + static_cast<int64_t>(q0) * k;
         p.out_logits = out_logits + static_cast<int64_t>(q0) * k;
         p.sparse = sparse != nullptr ? sparse + static_cast<int64_t>(q0) * head->V : nullptr;

@@ -22,7 +22,16 @@ constexpr bool bound_words_fit(int slots, int blocks) { return slots * blocks <=
 // where one will do: 12000 rows, 64 queries, k = 50: 32.5 us with one, 54.5 with
 // four); none (0) where the rows do not give k of them, which every launch
 // would wait for in vain.
-constexpr int tc_bound_blocks(int slots, int k, int G, int64_t V) {
+// None either where k is so small that a list fills in a handful of insertions
+// and starting all CTAs in step costs more: 64 slots at k = 1 (without / with the
+// bound: 262144 x 1152 106.5 / 109.7 us, 151936 x 1024 65.5 / 67.6), and up to
+// k = 3 where a row's `pitch` bytes are no multiple of a 32-byte sector, so that
+// each box of the query matrix, which CTAs in step read at once, takes more of
+// them (100003 x 1000, 64 queries: k = 1 57.8 / 68.4, k = 3 60.2 / 69.1, k = 8 68.7 /
+// 68.6; e4m3, 32 queries: 41.3 / 48.5, 43.9 / 48.6, 52 without at k = 8 / 48.7; the
+// 4-slot tile never waits for the bound and keeps it).
+constexpr int tc_bound_blocks(int slots, int k, int G, int64_t V, int64_t pitch) {
+    if ((slots == 64 && k == 1) || (slots > 4 && k <= 3 && pitch % 32 != 0)) return 0;
     const int b = 2 * k <= G || !bound_words_fit(slots, 4) ? 1 : 4;
     const int64_t blocks = b == 1 ? (V + 127) / 128 : (V + 31) / 32;  // words there can be
     const int64_t words = blocks < b * G ? blocks : b * G;

@@ -38,6 +38,8 @@ def test_plan_selects_paths(vie):
     (30011, 256, 40, 65),    # two 32-query groups, two queries per selector warp
     (20011, 1152, 100, 50),  # 64 + 36 queries
     (30011, 256, 32, 1),     # greedy, full group of 32
+    (30011, 1000, 64, 1),    # no shared bound: greedy on 64 slots, rows of odd sectors
+    (30011, 1000, 20, 3),
     (50021, 1024, 17, 77),
     (100, 64, 4, 50),        # one tile: most CTAs draw nothing and write empty lists
     (64, 128, 2, 64),        # k = V on one CTA
