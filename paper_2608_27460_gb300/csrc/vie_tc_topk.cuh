@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(TcShape<NQ, Q8>::kThreads, 1)
                 }
                 const int nst = tile < 0 ? 1 : n_st;
                 for (int st_i = 0; st_i < nst; ++st_i) {
-                    if (issued == S) griddep_wait();  // as for the MMA issuer's waits
+                    if (Q8 && hres && issued == S) griddep_wait();  // as for the MMA issuer's waits (else: below)
                     if (issued >= S && !mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
                         ok = false;
                         break;
