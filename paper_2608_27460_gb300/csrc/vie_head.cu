@@ -1118,7 +1118,7 @@ vie_status vie_head_device_status(vie_head *head, vie_stream stream) {
 namespace {
 
 constexpr size_t kNoAllocScratchBytes = size_t(1) << 20;  // 1 MiB per device
-constexpr size_t kNoAllocCounterBytes = 256;              // counters, then the lists
+constexpr size_t kNoAllocCounterBytes = 256;              // its last bytes: counters, behind the lists
 constexpr size_t kNoAllocBoundBytes = size_t(kMaxNB) * vie::kBoundMax * sizeof(uint64_t);  // behind them
 
 // Host code sees only a stand-in for this array; kernels get its device
@@ -1203,20 +1203,20 @@ extern "C" vie_status vie_head_topk_noalloc(const void *W_out, int64_t V, int32_
                     "smaller batch or k",
                     fn, lists_bytes, nb_max, G, k, vie::kFastE,
                     kNoAllocScratchBytes - kNoAllocCounterBytes);
-    uint64_t *cand = reinterpret_cast<uint64_t *>(nd.scratch + kNoAllocCounterBytes);
+    uint64_t *cand = reinterpret_cast<uint64_t *>(nd.scratch);
     uint64_t *heads = cand + list_keys;
     if ((reinterpret_cast<uintptr_t>(cand) | reinterpret_cast<uintptr_t>(heads)) & 15u)
         return fail(VIE_ERR_UNSUPPORTED, "%s: scratch lists not 16-byte aligned", fn);
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    uint32_t *counters = reinterpret_cast<uint32_t *>(nd.scratch);
-    e = cudaMemsetAsync(counters, 0, 4 * sizeof(uint32_t), s);  // ticket and pool start at 0
-    // the shared bounds' words: none left of another call, whose tags (the
-    // group's number) repeat
+    // One clear: ticket and pool start at 0, and of the shared bounds' words
+    // behind them none is left of another call, whose tags (the group's number)
+    // repeat (a second memset on the stream costs a call ~2 us).
+    uint32_t *counters = reinterpret_cast<uint32_t *>(nd.scratch + kNoAllocScratchBytes - kNoAllocCounterBytes);
     uint64_t *gmax = reinterpret_cast<uint64_t *>(nd.scratch + kNoAllocScratchBytes);
     const int gt_blocks = bound_blocks_for(k, V, G);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(gmax, 0, static_cast<size_t>(nb_max) * G * gt_blocks * sizeof(uint64_t), s);
+    e = cudaMemsetAsync(counters, 0,
+                        kNoAllocCounterBytes + static_cast<size_t>(nb_max) * G * gt_blocks * sizeof(uint64_t), s);
     if (e != cudaSuccess) return fail_cuda(e, "vie_head_topk_noalloc clear");
     for (int q0 = 0; q0 < batch; q0 += cap) {
         const int nq = batch - q0 < cap ? batch - q0 : cap;
