@@ -67,7 +67,8 @@ typedef struct {
     int32_t ctas;         /* CTAs of one projection launch (one per SM max)  */
     int32_t device;       /* CUDA device ordinal the handle lives on         */
     int64_t weight_bytes; /* bytes of the owned padded copy of W_out         */
-    int64_t scratch_bytes;/* bytes of per-handle scratch                      */
+    int64_t scratch_bytes;/* bytes of per-handle scratch, query matrix and all
+                             (not vie_head_topk_host's staging buffers)       */
 } vie_head_props;
 
 /*

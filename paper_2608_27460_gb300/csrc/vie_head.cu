@@ -58,7 +58,7 @@ constexpr int kEpochWord = 4;
 constexpr int kFlagWords = 8;
 constexpr int kCountWords = kFlagWords + vie::kMaxLists;
 constexpr int kNumWords = kCountWords + vie::kTcMaxSelWarps;
-// Rows of a bf16 head's query matrix: hi and lo of a block of many queries.
+// Rows of the query matrix of a head that takes many queries: hi and lo of a block of them.
 constexpr int kHRows = 2 * vie::kMnBlock;
 static_assert(kHRows >= vie::kTcHRows, "the batched path's query matrix fits");
 
@@ -77,7 +77,7 @@ struct vie_head {
     uint64_t *gmax;     // [G * vie::kBoundWords] maxima behind the shared bounds (tagged words), in cand's allocation
     int64_t scratch_bytes;
     // tensor-core path (batches): hi/lo bf16 query matrix and TMA descriptors
-    void *hB;             // [kHRows][d_pad] bf16, or e4m3 query pieces [4 NQ][d_pad]; in cand's allocation
+    void *hB;             // [kHRows or kTcHRows][d_pad] bf16, or e4m3 query pieces [4 NQ][d_pad]; in cand's allocation
     float *qscale;        // e4m3 heads: [32][kQ8Pieces] piece scales of the query group
     bool tc_ready;
     CUtensorMap mapW;     // W as [V][d_pad], box 128 rows x 128 bytes, 128-byte swizzle
@@ -376,11 +376,16 @@ int many_block(const vie_head *hd, int k) {
     return static_cast<int>(n < vie::kMnBlock ? n : vie::kMnBlock);
 }
 
+// Whether a head can take many queries at once (and needs their query matrix).
+bool many_possible(const vie_head *hd, bool e4m3) {
+    return !e4m3 && hd->V >= kManyMinRows && hd->d_pad >= 64 && hd->num_sms >= 2 &&
+           hd->cand_bytes >= vie::kMnBlock * vie::kMnCap * sizeof(uint64_t);
+}
+
 // Sets up a bf16 head for many queries, in scratch that the other paths use
 // between such calls.
 void init_many(vie_head *hd) {
-    hd->many_ready = hd->tc_ready && hd->V >= kManyMinRows && hd->d_pad >= 64 && hd->num_sms >= 2 &&
-                     hd->cand_bytes >= vie::kMnBlock * vie::kMnCap * sizeof(uint64_t);
+    hd->many_ready = hd->tc_ready && many_possible(hd, false);
     const uint64_t pitch = static_cast<uint64_t>(hd->d_pad) * 2;
     if (hd->many_ready) hd->many_ready = make_map_bf16(&hd->mapHM, hd->hB, kHRows, hd->d_pad, pitch, 128);
     for (int i = 0; i < 4 && hd->many_ready; ++i) {
@@ -467,13 +472,14 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
     const size_t gbytes = static_cast<size_t>(hd->G) * vie::kBoundWords * sizeof(uint64_t);
     const size_t mbytes = static_cast<size_t>(vie::kMnBlock) * (sizeof(uint64_t) + 3 * sizeof(uint32_t));
     hd->cand_bytes = cbytes;
-    hd->scratch_bytes = static_cast<int64_t>(cbytes + gbytes + mbytes + kNumWords * sizeof(uint32_t));
     e = cudaMalloc(&hd->W, wbytes);
     if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->scale, static_cast<size_t>(V) * sizeof(float));
     // one allocation and one clear: tagged words of no launch (tag 0), empty
     // lists until written, zero query rows
     const size_t hoff = (cbytes + gbytes + mbytes + 255) & ~static_cast<size_t>(255);
-    const size_t hbytes = static_cast<size_t>(e4m3 ? vie::kTcHRows : kHRows) * hd->d_pad * 2;
+    const size_t hbytes = static_cast<size_t>(many_possible(hd, e4m3) ? kHRows : vie::kTcHRows) * hd->d_pad * 2;
+    const size_t qbytes = e4m3 ? 32 * vie::kQ8Pieces * sizeof(float) : 0;
+    hd->scratch_bytes = static_cast<int64_t>(hoff + hbytes + qbytes + kNumWords * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMalloc(&hd->cand, hoff + hbytes);
     if (e == cudaSuccess) e = cudaMemset(hd->cand, 0, hoff + hbytes);
     if (e == cudaSuccess) {
@@ -481,7 +487,7 @@ static vie_status create_head(const void *W_out, int64_t V, int32_t d, vie_dtype
         hd->hB = reinterpret_cast<unsigned char *>(hd->cand) + hoff;
     }
     if (e == cudaSuccess) e = cudaMalloc(&hd->words, kNumWords * sizeof(uint32_t));
-    if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->qscale, 32 * vie::kQ8Pieces * sizeof(float));
+    if (e == cudaSuccess && e4m3) e = cudaMalloc(&hd->qscale, qbytes);
     if (e == cudaSuccess) e = cudaMemset(hd->words, 0, kNumWords * sizeof(uint32_t));
     if (e == cudaSuccess && e4m3) {
         int64_t blocks = (V + 7) / 8;  // 8 rows (warps) per block

@@ -13,6 +13,25 @@ from paper_2608_27460_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("storage", ["bf16", "e4m3"])
+@pytest.mark.parametrize("V,d", [(8000, 16384), (8192, 8192), (20011, 48)])
+def test_handle_memory_is_what_its_props_say(vie, storage, V, d):
+    """Weights and scratch of a handle, the query matrix with it: for 512 queries
+    only where a call can take that many at once (bf16, V >= 8192, d >= 64)."""
+    import torch
+    W = torch.zeros((V, d), dtype=torch.int16, device="cuda")
+    vie.Head(W, storage=storage).close()  # the kernels' own memory is there now
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    with vie.Head(W, storage=storage) as head:
+        used = before - torch.cuda.mem_get_info()[0]
+        p = head.props
+        rows = 1024 if storage == "bf16" and V >= 8192 and d >= 64 else 128
+        assert p.scratch_bytes >= rows * p.d_pad * 2
+        assert p.scratch_bytes <= rows * p.d_pad * 2 + p.ctas * (8 * 1056 + 256) * 8 + (64 << 10)
+        assert used <= p.weight_bytes + p.scratch_bytes + (10 << 20)  # whole 2 MB pages
+
+
 def test_plan_selects_paths(vie):
     W, _ = workload(20011, 640, 1, seed=3)
     with vie.Head(to_device_bits(W)) as head:
