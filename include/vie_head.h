@@ -378,7 +378,7 @@ vie_status vie_scatter_sparse_logits(const int32_t *idx, const float *logits, in
  *         while cap * c * 8 > 32768, where c = max(256, 2k rounded up to a
  *         multiple of 64) is the candidate buffer of one query.
  * Scratch: one 1 MiB array per device (every GPU that loads the library keeps
- * it until the process exits), of which the first 256 bytes hold counters, and
+ * it until the process exits), of which the last 256 bytes hold counters, and
  * 80 KiB behind it for the bounds that the CTAs of a launch share.
  * A call needs
  *   8 * (round_up_even(slots * ctas * k) + slots * ctas * 8)

@@ -30,6 +30,7 @@ pytestmark = pytest.mark.gpu
     (5000, 64, 3, 3),        # 4 slots x 79 x 3: even, three queries
     (30011, 64, 3, 150),     # wide lists: 320-key candidate buffers, 4 slots
     (30011, 64, 1, 600),     # wide lists, one 1216-key buffer
+    (6000, 640, 2, 128),     # wide lists of 64 rows per CTA: no shared bound
 ])
 def test_noalloc_matches_oracle_and_head_topk_twice(vie, V, d, batch, k):
     import torch
