@@ -43,12 +43,12 @@ PROFILE_DIR = os.path.join(ROOT, "profiles")
 # the digest of these files, and its traffic figure is used only while the
 # digest still matches.
 KERNEL_SOURCES = {
-    "stream_topk": ["vie_stream_topk.cuh", "vie_device.cuh", "vie_stream_topk_inst.cuh"],
-    "stream_topk_e4m3": ["vie_stream_topk.cuh", "vie_device.cuh", "vie_stream_topk_inst.cuh"],
+    "stream_topk": ["vie_stream_topk.cuh", "vie_device.cuh", "vie_plan.h", "vie_stream_topk_inst.cuh"],
+    "stream_topk_e4m3": ["vie_stream_topk.cuh", "vie_device.cuh", "vie_plan.h", "vie_stream_topk_inst.cuh"],
     "tc_topk": ["vie_tc_topk.cuh", "vie_tc_topk.cu", "vie_tc_launch.cuh", "vie_tcgen05.cuh", "vie_device.cuh",
-                "vie_stream_topk.cuh"],
+                "vie_plan.h", "vie_stream_topk.cuh"],
     "tc_topk_e4m3": ["vie_tc_topk.cuh", "vie_tc_topk_e4m3.cu", "vie_tc_launch.cuh", "vie_tcgen05.cuh",
-                     "vie_device.cuh", "vie_stream_topk.cuh"],
+                     "vie_device.cuh", "vie_plan.h", "vie_stream_topk.cuh"],
 }
 
 

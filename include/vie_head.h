@@ -132,12 +132,15 @@ vie_status vie_head_destroy(vie_head *head);
 /* Fills *props (host) with the handle's facts. */
 vie_status vie_head_get_props(const vie_head *head, vie_head_props *props);
 
-/* How a vie_head_topk / vie_head_topk_sparse call of this size runs.  (bf16
- * batches of 256 queries or more with k <= 128 run as a filtered GEMM on the
- * tensor cores: groups of 128 queries, five launches per block of up to 512.) */
+/* How a vie_head_topk / vie_head_topk_sparse call of this size runs.  Each
+ * query group is one pass over W_out, but for bf16 batches of 256 queries or
+ * more with k <= 128 (on vocabularies of 8192 rows or more whose sample fits the
+ * handle's scratch): those run as a filtered GEMM on the tensor cores, in groups
+ * of 128 queries, and read W_out about once per block of up to four groups (plus
+ * every 8th to 64th row), five launches each: launches / 5 times. */
 typedef struct {
     int32_t path;     /* 0: streaming CUDA-core kernel, 1: tensor-core kernel  */
-    int32_t groups;   /* query groups, one pass over W_out each               */
+    int32_t groups;   /* query groups (see above)                             */
     int32_t launches; /* kernel launches the call enqueues                    */
 } vie_topk_plan;
 
@@ -202,6 +205,10 @@ vie_status vie_get_launch_option(vie_launch_option option, int32_t *value);
  *               the bf16 x fp32 products).
  *   stream      the stream the work is enqueued on.
  *
+ * Batches on the tensor cores start by sharing a bound on the k-th logit
+ * between all CTAs of the launch, one per SM, and wait at most 20 us for it; when
+ * kernels of another stream hold some SMs, that wait runs out on every such
+ * launch (the results are the same).
  * The full logit vector is never written to memory.  Calls using the same
  * handle share its scratch, so at most one vie_head_topk per handle may be
  * in flight at a time (calls on one stream are naturally serialised).

@@ -358,9 +358,13 @@ bool make_map_bf16(CUtensorMap *m, void *base, uint64_t rows, uint64_t cols, uin
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Batches of at least this many queries run as a filtered GEMM.  Below it the
-// batched path's passes over W (64 queries each) cost less than a block's five
-// launches and its sample.
+// Batches of at least this many queries run as a filtered GEMM.  The line is not
+// where the two cost the same: from 65 queries on the filtered GEMM is the faster
+// one but on small vocabularies with larger k (passes / filtered GEMM, us, k = 2:
+// 151936 x 1024 65 queries 122 / 76, 128 137 / 78, 255 274 / 119; 128256 x 3072 65
+// 258 / 160, 128 265 / 166, 255 531 / 270; 20011 x 640 65 55 / 48, 255 135 / 53; k = 50:
+// 151936 x 1024 65 125 / 108, 128 141 / 109; 20011 x 640 65 57 / 94, 128 71 / 83, 255 141 /
+// 114).  Moving it is a change of route of its own and has not been made.
 constexpr int kManyMinBatch = 256;
 constexpr int64_t kManyMinRows = 8192;  // a smaller vocabulary's sample bounds too little
 

@@ -647,8 +647,9 @@ static __device__ __noinline__ int warp_filter(uint64_t *buf, int cnt, uint64_t 
     return base;
 }
 
-// The same for k <= kFastMaxK (streams too short for the shared bound): every key of the buffer (at most kSelCapFast) is ranked by counting the keys
-// above it, one thread per key, and the best k go out at their rank (~1.5 us
+// As write_cta_list for k <= kFastMaxK (streams too short for the shared
+// bound): every key of the buffer (at most kSelCapFast) is ranked by counting the
+// keys above it, one thread per key, and the best k go out at their rank (~1.5 us
 // for 224 keys).
 __device__ inline void write_ranked_list(const uint64_t *buf, int cnt, int k, uint64_t *dst, uint64_t *head) {
     const int tid = threadIdx.x, nthr = static_cast<int>(blockDim.x);
@@ -1348,7 +1349,7 @@ __device__ __forceinline__ float fma_e4m3x4(uint32_t w, float4 h, float a) {
 
 // The launch may overlap the kernel before it on the stream (p.pdl: programmatic
 // dependent launch): a CTA starts as soon as an SM frees up, and its producer
-// fills the ring with W (constant while the handle lives) while the previous
+// requests one stage of W (constant while the handle lives) while the previous
 // launch still merges; everything else waits for that launch's completion.
 // Back to back this hides the ramp of the stream and the merge: 51.4 -> 49.0 us
 // per step at V = 151936, d = 1024, 26.4 -> 22.4 us at V = 20011, d = 640.

@@ -5,8 +5,9 @@
 // Per block of up to kMnBlock queries, five launches:
 //   prep    the hi/lo bf16 query matrix (as on the batched path);
 //   sample  the GEMM below on every s-th row of W, logits written out;
-//   tau     per query, the k-th largest key of the sample (exact): a bound on
-//           the k-th key of the whole vocabulary;
+//   tau     per query, a key with at least k sampled keys at or above it (the
+//           k-th largest, or one of little higher rank): a bound on the k-th
+//           key of the whole vocabulary;
 //   main    the GEMM on all rows; a logit whose key is at least the query's
 //           tau is appended to its candidate list (about k s of them, s chosen
 //           so that kMnCap holds them), everything else stays on the chip;
@@ -14,9 +15,9 @@
 // The sample takes every s-th row of the total order's index range, and tau is
 // a key (logit, then row), so neither ties nor clusters of neighbouring rows
 // make many candidates; a query whose list overflows all the same (kMnCap)
-// is recomputed from all rows by the CTAs of the final launch.  20000 queries, 151936 x 1024,
-// k = 2: 22.0 ms in passes of 64 queries, 9.1 ms here (per 512 queries: main
-// 194 us, 1.64 PFLOP/s; the other four launches ~30 us).
+// is recomputed from all rows by the CTAs of the final launch.  20000 queries,
+// 151936 x 1024, k = 2: 22.0 ms in passes of 64 queries, 9.0 ms here (per 512
+// queries: main 194 us, 1.64 PFLOP/s; the other four launches ~30 us).
 //
 // The GEMM runs on CTA pairs (tcgen05 cta_group::2): M = 256 rows of W, half
 // per CTA, times N = 256 columns, 128 queries as hi and lo. Each CTA stages its

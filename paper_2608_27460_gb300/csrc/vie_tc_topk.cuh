@@ -31,7 +31,10 @@
 //                (at most kTcBoundWaitNs) before the first tile is entered;
 //                a few keys per query and CTA are left (128256 x 3072, k = 50:
 //                159.9 -> 140.1 us at 64 queries; e4m3 82.4 -> 74.5 us at 16,
-//                115.7 -> 83.3 us at 32).
+//                115.7 -> 83.3 us at 32; where it is used: tc_bound_blocks).
+//                A launch whose CTAs cannot all start at once, because kernels
+//                of another stream hold SMs, waits its full limit and goes on
+//                with the bound it has.
 // Each CTA writes its per-query lists and takes a completion ticket; the
 // last CTAs to finish merge them, one query each.  All waits are bounded.
 //
