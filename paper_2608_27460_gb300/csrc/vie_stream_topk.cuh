@@ -1121,10 +1121,13 @@ __device__ inline void merge_queries(const uint64_t *cand, const uint64_t *heads
 // keys) are merged in full.  ws holds the merge buffers (merge_fixed_bytes);
 // fe holds G * kFastE keys and then ceil(G/8)*8 head words.  Every wait is
 // bounded; a list that never arrives is reported in *err and nothing is written.
-__device__ inline void merge_published(const uint32_t *flags, uint32_t target, const uint64_t *heads_q,
-                                       const uint64_t *lists_q, int G, int k, unsigned char *ws,
-                                       uint64_t *fe, MiscSmem *ms, uint32_t *err, int32_t *oi, float *ol,
-                                       float *sp) {
+// (This and the next out of line: inlined, they and the selectors took 168
+// registers in the one-query kernel and spilled in the eight-query one.  A step on an
+// idle GPU with a cold L2: 128256 x 2048, b = 1, k = 1 82.7 -> 81.9 us.)
+static __device__ __noinline__ void merge_published(const uint32_t *flags, uint32_t target,
+                                                    const uint64_t *heads_q, const uint64_t *lists_q, int G, int k,
+                                                    unsigned char *ws, uint64_t *fe, MiscSmem *ms, uint32_t *err,
+                                                    int32_t *oi, float *ol, float *sp) {
     const int tid = threadIdx.x;
     MergeBufs mb;
     mb.pref = reinterpret_cast<uint64_t *>(ws);
@@ -1177,18 +1180,6 @@ __device__ inline void merge_published(const uint32_t *flags, uint32_t target, c
     const bool fast_ok = k <= G && 2 * G <= static_cast<int>(blockDim.x);
     if (!(fast_ok && merge_fast_query(fe, hv, G, k, mb.cands, mb.counts, ms, oi, ol, sp)))
         merge_lists(GlobalKeys{lists_q}, G, k, mb, ms, oi, ol, sp);
-}
-
-// The same out of line, for the streaming kernel: inlined, this merge, the next
-// and the selectors took 168 registers with one query and spilled with eight.  A
-// step on an idle GPU with a cold L2: 128256 x 2048, b = 1, k = 1 82.7 -> 81.9 us.
-// (The tensor-core kernel keeps it inline: 96.8 us inline, 97.9 out of line at
-// 262144 x 1152, b = 4, alone; 91.9 and 92.2 behind one another.)
-static __device__ __noinline__ void merge_published_call(const uint32_t *flags, uint32_t target,
-                                                         const uint64_t *heads_q, const uint64_t *lists_q, int G,
-                                                         int k, unsigned char *ws, uint64_t *fe, MiscSmem *ms,
-                                                         uint32_t *err, int32_t *oi, float *ol, float *sp) {
-    merge_published(flags, target, heads_q, lists_q, G, k, ws, fe, ms, err, oi, ol, sp);
 }
 
 // Merge of one query from published wide lists (k > kFastMaxK; every thread
@@ -1823,7 +1814,7 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
         if (tid == 0) st_release_gpu(p.flags + cta, target);
         if (cta != 0) return;
         unsigned char *ws = smem + L.merge;
-        merge_published_call(p.flags, target, p.heads, p.cand, G, p.k, ws,
+        merge_published(p.flags, target, p.heads, p.cand, G, p.k, ws,
                         reinterpret_cast<uint64_t *>(ws + SmemLayout::merge_fixed_bytes()), ms, p.err,
                         p.out_idx, p.out_logits, p.sparse);
         if (tid == 0) {
@@ -1867,7 +1858,7 @@ __global__ void __launch_bounds__(threads_for<NB>(), 1) stream_topk_kernel(const
                                      p.cand + static_cast<size_t>(q) * G * p.list_keys, p.list_keys, G, p.k, ws,
                                      fe, ms, p.err, oi, ol, sp);
             else
-                merge_published_call(p.flags, target, p.heads + static_cast<size_t>(q) * G * kFastE,
+                merge_published(p.flags, target, p.heads + static_cast<size_t>(q) * G * kFastE,
                                 p.cand + static_cast<size_t>(q) * G * p.k, G, p.k, ws, fe, ms, p.err, oi, ol, sp);
             __syncthreads();
         }
