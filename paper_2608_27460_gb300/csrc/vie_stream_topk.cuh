@@ -1121,13 +1121,10 @@ __device__ inline void merge_queries(const uint64_t *cand, const uint64_t *heads
 // keys) are merged in full.  ws holds the merge buffers (merge_fixed_bytes);
 // fe holds G * kFastE keys and then ceil(G/8)*8 head words.  Every wait is
 // bounded; a list that never arrives is reported in *err and nothing is written.
-// (This and the next out of line: inlined, they and the selectors took 168
-// registers in the one-query kernel and spilled in the eight-query one.  A step on an
-// idle GPU with a cold L2: 128256 x 2048, b = 1, k = 1 82.7 -> 81.9 us.)
-static __device__ __noinline__ void merge_published(const uint32_t *flags, uint32_t target,
-                                                    const uint64_t *heads_q, const uint64_t *lists_q, int G, int k,
-                                                    unsigned char *ws, uint64_t *fe, MiscSmem *ms, uint32_t *err,
-                                                    int32_t *oi, float *ol, float *sp) {
+__device__ inline void merge_published(const uint32_t *flags, uint32_t target, const uint64_t *heads_q,
+                                       const uint64_t *lists_q, int G, int k, unsigned char *ws,
+                                       uint64_t *fe, MiscSmem *ms, uint32_t *err, int32_t *oi, float *ol,
+                                       float *sp) {
     const int tid = threadIdx.x;
     MergeBufs mb;
     mb.pref = reinterpret_cast<uint64_t *>(ws);
@@ -1196,11 +1193,10 @@ static __device__ __noinline__ void merge_published(const uint32_t *flags, uint3
 //      key >= tau is gathered from the whole lists (lists_q, G x list_keys,
 //      unsorted, zeros as empty slots).
 // ws holds the merge buffers (merge_fixed_bytes), fe G * (kWideE + 1) keys.
-static __device__ __noinline__ void merge_published_wide(const uint32_t *flags, uint32_t target,
-                                                         const uint64_t *heads_q, const uint64_t *lists_q,
-                                                         int list_keys, int G, int k, unsigned char *ws, uint64_t *fe,
-                                                         MiscSmem *ms, uint32_t *err, int32_t *oi, float *ol,
-                                                         float *sp) {
+__device__ inline void merge_published_wide(const uint32_t *flags, uint32_t target, const uint64_t *heads_q,
+                                            const uint64_t *lists_q, int list_keys, int G, int k,
+                                            unsigned char *ws, uint64_t *fe, MiscSmem *ms, uint32_t *err,
+                                            int32_t *oi, float *ol, float *sp) {
     const int tid = threadIdx.x, lane = tid & 31, nthr = static_cast<int>(blockDim.x);
     MergeBufs mb;
     mb.pref = reinterpret_cast<uint64_t *>(ws);
