@@ -693,6 +693,40 @@ struct MergeBufs {
     uint32_t *hist;
 };
 
+// The best k of n unique nonzero keys in shared memory, written best first: a
+// radix select first if they are many, then ranked by all pairs, or sorted.  Out
+// of line: block_topk_to_output seldom needs it.  (hist may hold what the caller
+// has just read: a barrier comes first.)
+static __device__ __noinline__ void rank_crowded(uint64_t *keys, int n, int k, uint64_t *win, uint32_t *hist,
+                                                 MiscSmem *ms, int32_t *out_idx, float *out_logits,
+                                                 float *sparse_row) {
+    const int tid = threadIdx.x, nthr = static_cast<int>(blockDim.x);
+    uint64_t *src = keys;
+    int m = n;
+    __syncthreads();
+    if (n > kRankCountMax && n > k) {
+        const uint64_t T = block_radix_threshold(SmemKeys{keys}, n, k, 1, hist, ms);
+        if (tid == 0) ms->n_win = 0;
+        __syncthreads();
+        for (int i = tid; i < n; i += nthr)
+            if (keys[i] >= T) win[atomicAdd(&ms->n_win, 1)] = keys[i];
+        __syncthreads();
+        src = win;
+        m = k;
+    }
+    if (m > kRankCountMax) block_sort_desc(src, m);  // (room for the power of two above in either)
+    for (int i = tid; i < m; i += nthr) {
+        const uint64_t x = src[i];
+        const int rank = m > kRankCountMax ? i : rank_among(src, m, x);
+        if (rank < k) {
+            out_idx[rank] = key_index(x);
+            out_logits[rank] = key_value(x);
+            if (sparse_row != nullptr) sparse_row[key_index(x)] = key_value(x);
+        }
+    }
+    __syncthreads();
+}
+
 // Exact top-k of n (at most kMergeCandCap) unique nonzero keys in shared
 // memory (not mb.pref), written best first to out_idx / out_logits (and into
 // the sparse row, if any).  A counting sort by logit: the keys' range of
@@ -778,32 +812,8 @@ __device__ inline void block_topk_to_output(const uint64_t *keys, int n, int k, 
         }
     }
     __syncthreads();
-    const bool crowded = range[2] != 0;
-    if (crowded) {
-        __syncthreads();  // `range` has been read: the radix select uses its memory
-        uint64_t *src = sorted;
-        int m = n;
-        if (n > kRankCountMax && n > k) {
-            const uint64_t T = block_radix_threshold(SmemKeys{sorted}, n, k, 1, mb.hist, ms);
-            if (tid == 0) ms->n_win = 0;
-            __syncthreads();
-            for (int i = tid; i < n; i += nthr)
-                if (sorted[i] >= T) mb.win[atomicAdd(&ms->n_win, 1)] = sorted[i];
-            __syncthreads();
-            src = mb.win;
-            m = k;
-        }
-        if (m > kRankCountMax) block_sort_desc(src, m);  // (room for the power of two above in either)
-        for (int i = tid; i < m; i += nthr) {
-            const uint64_t x = src[i];
-            const int rank = m > kRankCountMax ? i : rank_among(src, m, x);
-            if (rank < k) {
-                out_idx[rank] = key_index(x);
-                out_logits[rank] = key_value(x);
-                if (sparse_row != nullptr) sparse_row[key_index(x)] = key_value(x);
-            }
-        }
-        __syncthreads();
+    if (range[2] != 0) {
+        rank_crowded(sorted, n, k, mb.win, mb.hist, ms, out_idx, out_logits, sparse_row);
         return;
     }
     for (int i = tid; i < n; i += nthr) {
